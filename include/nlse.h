@@ -167,15 +167,16 @@ nlse_status nlse_alu_probe(int32_t kind, int32_t iters, int32_t blocks, void* cu
 
 /* Column tile of the column pass: a width of 1, 2, 4, 8 or 16 columns per
  * block, or'ed with NLSE_COL_TMA for the variant that moves the tile between
- * global and shared memory with bulk tensor copies (cp.async.bulk.tensor,
- * boxes of 512 rows) instead of per-thread loads and stores (n >= 512), and
+ * global and shared memory with bulk tensor copies (cp.async.bulk.tensor)
+ * instead of per-thread loads and stores (n >= 512), and
  * in FP32 with NLSE_COL_R8 for the radix-8 column transform (8 elements per
  * thread, more threads in flight, one more shared-memory exchange; radix 16
  * without it).  The field between the passes is stored in 16-byte units that
  * hold one column's values at two adjacent rows, so a column is a sequence of
  * units.  NLSE_EUNSUPPORTED for a tile this size or precision cannot use.
- * Chosen by the autotuner (default FP32: the narrowest radix-16 staged tile
- * of at least 128 threads); for a given radix the results do not depend on
+ * Chosen by the autotuner (default FP32: radix-16 staged pairs of columns for
+ * n = 512..4096, staged single columns for n = 8192, narrow per-thread tiles
+ * below, radix 8 for n <= 128); for a given radix the results do not depend on
  * the tile, bit for bit, while the radix changes the rounding (both stay
  * within the stated tolerances).  A bounded wait (1 s) of the staged variant
  * that runs out makes the block skip its tile and sets NLSE_ETIMEOUT in the
@@ -188,10 +189,11 @@ enum { NLSE_COL_TMA = 0x100, NLSE_COL_R8 = 0x200 };
 nlse_status nlse_set_column_tile(nlse_grid* g, int32_t cols);
 
 /* Radix of the row pass's transforms: 16 (16 elements per thread, the default
- * in FP32) or 8 (8 elements per thread: twice the threads in flight, one more
- * shared-memory exchange per transform); FP64 grids take 8 only.
- * NLSE_ROW_STAGED | 16 (FP32, n >= 2048): radix 16 with persistent blocks, each
- * moving its next row pair into shared memory with one bulk copy while it
+ * in FP32 for n = 256..4096) or 8 (8 elements per thread: twice the threads in
+ * flight, one more shared-memory exchange per transform; the default for
+ * n <= 128); FP64 grids take 8 only.
+ * NLSE_ROW_STAGED | 16 (FP32, n >= 2048, the default for n = 8192): radix 16 with persistent blocks, each
+ * moving its next row pair into shared memory with bulk copies while it
  * finishes the current one; bit-identical to radix 16, its wait for a copy
  * bounded as the staged column pass's (NLSE_ETIMEOUT, see
  * nlse_set_column_tile).  NLSE_EUNSUPPORTED otherwise.  Chosen by the

@@ -46,8 +46,8 @@ struct BatchBeam {
     const float2* px;  // kDitherP copies of n entries each (copy k mod kDitherP serves step k)
     const unsigned char* py;  // kDitherP copies of P_y and the cross-lane factors (py32_copy_bytes)
     const unsigned char* tw;  // kDither twiddle blocks (pass32.cuh: tw32_copy_bytes)
-    const CUtensorMap* map;   // the field as n/2 row pairs x n columns x 4 words, boxes of one
-                              // column x 256 row pairs (staged column tiles; null for n < 512)
+    const CUtensorMap* map;   // the field as n/2 row pairs x 4 n words (pass32.cuh: p_col_il,
+                              // p_col_box_rows; null for n < 512)
     ScreenCoef<float> sc;
     int log2n;
     int col_tiles;
@@ -124,8 +124,8 @@ struct StageState {
 
 // One staged column tile (beam with n >= 512): thread 0 orders the rows other
 // blocks wrote (acquired through the completion counter) before its bulk
-// copies, moves the C columns into their transform lines with one box of 256
-// row pairs per copy and waits for them, bounded; every thread transforms its
+// copies, moves the C columns into their transform lines (pass32.cuh:
+// col_stage_load) and waits for them, bounded; every thread transforms its
 // column exactly as col_tile32 does; thread 0 stores the lines back with bulk
 // copies and waits until those writes are complete, so that the completion
 // signal that follows covers them.  On a wait that runs out the block records
@@ -135,20 +135,15 @@ template <int THREADS, int E, int N>
 __device__ __forceinline__ bool batch_col_staged(const BatchBeam& bm, int tile, const unsigned char* twb,
                                                  const float2* px, const float4* py, float2 rot, C2* smem,
                                                  StageState& st, const BatchPlan& plan) {
-    constexpr int L = N / 2, EE = p_e<L, E>(), T = p_col_tpl<N, E>(), C = tile_cols<THREADS, E, N>();
-    constexpr int LS = pr::pair_line_stride<L, EE, C>(), BOXES = L / kTmaBoxRows;
-    constexpr uint32_t BYTES = (uint32_t)(C * L * 16);
+    constexpr int C = tile_cols<THREADS, E, N>();
+    constexpr uint32_t BYTES = (uint32_t)(C * (N / 2) * 16);
     const int col0 = tile * C;
     if (threadIdx.x == 0) {
         int fail = 0;
         fence_proxy_async_global();  // the acquired rows, before the copies read them
         fence_proxy_async_smem();    // this block's earlier use of the lines, before the copies write them
         mbar_expect_tx(st.bar, BYTES);
-#pragma unroll 1
-        for (int c = 0; c < C; ++c)
-#pragma unroll 1
-            for (int b = 0; b < BOXES; ++b)
-                tma_load_3d(smem + c * LS + b * kTmaBoxRows, bm.map, 0, col0 + c, b * kTmaBoxRows, st.bar);
+        col_stage_load<N, E, C>(smem, bm.map, col0, st.bar);
         if (!mbar_wait_bounded(st.bar, st.parity)) {
             atomicOr(plan.status, 2);
             atomicExch(plan.abort, 1);
@@ -160,23 +155,11 @@ __device__ __forceinline__ bool batch_col_staged(const BatchBeam& bm, int tile, 
     }
     __syncthreads();
     if (*st.fail) return false;  // (uniform)
-    const int c = (int)threadIdx.x / T, j = (int)threadIdx.x % T;
-    C2* line = smem + c * LS;
-    C2 v[EE];
-#pragma unroll
-    for (int m = 0; m < EE; ++m) v[m] = line[j + m * T];
-    __syncthreads();  // the staged tile is consumed; the transforms reuse its memory
-    col_body32<N, E>(v, line, twb, px, py, rot, col0 + c, j);
-#pragma unroll
-    for (int m = 0; m < EE; ++m) line[j + m * T] = v[m];
+    col_lines32<N, E, C>(smem, twb, px, py, rot, col0, threadIdx.x);
     fence_proxy_async_smem();
     __syncthreads();
     if (threadIdx.x == 0) {
-#pragma unroll 1
-        for (int cc = 0; cc < C; ++cc)
-#pragma unroll 1
-            for (int b = 0; b < BOXES; ++b)
-                tma_store_3d(bm.map, 0, col0 + cc, b * kTmaBoxRows, smem + cc * LS + b * kTmaBoxRows);
+        col_stage_store<N, E, C>(smem, bm.map, col0);
         tma_store_commit_and_wait();
         fence_proxy_async_global();  // the copies' writes, before the completion signal
     }
@@ -328,6 +311,22 @@ template <int THREADS, int E> int tiles_for(int log2n, bool col) {
     return 0;
 }
 
+// columns per box of the staged column tiles
+template <int THREADS, int E> int box_cols_for(int log2n) {
+    auto f = [&](auto nc) -> int {
+        constexpr int N = decltype(nc)::value;
+        if constexpr (batch_supported<THREADS, E, N>()) return p_col_il<N, E, tile_cols<THREADS, E, N>()>();
+        else return 1;
+    };
+    switch (log2n) {
+        case 9: return f(std::integral_constant<int, 512>{});
+        case 10: return f(std::integral_constant<int, 1024>{});
+        case 11: return f(std::integral_constant<int, 2048>{});
+        case 12: return f(std::integral_constant<int, 4096>{});
+    }
+    return 1;
+}
+
 struct BLayout {
     std::vector<size_t> field, px, py;
     size_t tw[kBatchMaxLog2 + 1];
@@ -353,7 +352,7 @@ BLayout blayout(int count, const nlse_params* ps) {
     for (int k = kBatchMinLog2; k <= kBatchMaxLog2; ++k) {
         bool used = false;
         for (int b = 0; b < count; ++b) used |= ps[b].n == (1 << k);
-        if (used) { L.tw[k] = o; o = al256(o + (size_t)kDither * tw32_copy_bytes(1 << k)); }
+        if (used) { L.tw[k] = o; o = al256(o + tw32_region_bytes(1 << k)); }
     }
     L.maps = o;      o = al256(o + sizeof(CUtensorMap) * count);  // 64-byte aligned each
     L.beams = o;     o = al256(o + sizeof(BatchBeam) * count);
@@ -387,7 +386,7 @@ nlse_status bvalidate(int count, const nlse_params* ps) {
 struct nlse_batch {
     int count;
     std::vector<nlse_params> ps;
-    std::vector<int> log2n, col_tiles, row_tiles;
+    std::vector<int> log2n, col_tiles, row_tiles, box_cols;
     cudaStream_t stream;
     unsigned char* ws;
     BLayout lay;
@@ -410,6 +409,7 @@ template <int THREADS, int E> nlse_status plan_tiles(nlse_batch* B) {
         if (tc == 0 || tr == 0) return NLSE_EUNSUPPORTED;
         B->col_tiles[b] = tc;
         B->row_tiles[b] = tr;
+        B->box_cols[b] = box_cols_for<THREADS, E>(B->log2n[b]);
     }
     B->smem = batch_smem_max<THREADS, E>();
     return NLSE_OK;
@@ -531,6 +531,7 @@ nlse_status nlse_batch_create(int32_t count, const nlse_params* params, const nl
     B->log2n.resize(count);
     B->col_tiles.resize(count);
     B->row_tiles.resize(count);
+    B->box_cols.resize(count);
     for (int b = 0; b < count; ++b) B->log2n[b] = ilog2i(params[b].n);
     B->stream = static_cast<cudaStream_t>(cuda_stream);
     B->ws = static_cast<unsigned char*>(dev_workspace);
@@ -564,7 +565,8 @@ nlse_status nlse_batch_create(int32_t count, const nlse_params* params, const nl
         d.tw = B->ws + lay.tw[B->log2n[b]];
         d.map = nullptr;
         if (params[b].n >= 2 * kTmaBoxRows) {
-            if (encode_field_map(&maps[b], d.field, params[b].n, 4, 1) != cudaSuccess) {
+            if (encode_unit_map(&maps[b], d.field, params[b].n, B->box_cols[b], p_col_box_rows(params[b].n, tn.radix)) !=
+                cudaSuccess) {
                 delete B;
                 return NLSE_ECUDA;
             }

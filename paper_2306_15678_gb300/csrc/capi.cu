@@ -41,9 +41,9 @@ size_t py_bytes(int n, int precision) {
     return precision == NLSE_FP64 ? (size_t)n * 16 : (size_t)kDitherP * py32_copy_bytes(n);
 }
 // bytes of the twiddle region: FP64 one pass-major table of n 16-byte
-// entries; FP32 kDither twiddle blocks (pass32.cuh: tw32_copy_bytes)
+// entries; FP32 kDither twiddle blocks and the one-off table (pass32.cuh)
 size_t tw_region_bytes(int n, int precision) {
-    return precision == NLSE_FP64 ? (size_t)n * 16 : (size_t)kDither * tw32_copy_bytes(n);
+    return precision == NLSE_FP64 ? (size_t)n * 16 : tw32_region_bytes(n);
 }
 
 int log2_exact(int n) {
@@ -223,8 +223,8 @@ int dither_offset(uint64_t table_id, uint64_t entry, int comp, int copies = kDit
 }
 // identifiers of the dithered tables (distinct offsets per table)
 enum : uint64_t {
-    kTabTwiddle = 1, kTabPx = 2, kTabPy = 3, kTabRowPair = 4, kTabColPair = 5, kTabCross = 6, kTabRowPair8 = 7,
-    kTabColPair8 = 8
+    kTabTwiddle = 1, kTabPx = 2, kTabPy = 3, kTabRowPair = 4, kTabCross = 6, kTabRowPair8 = 7, kTabColPair8 = 8,
+    kTabRowFused = 9, kTabColFused = 10
 };
 
 // Threshold of copy d (of `copies`, a power of two) for an entry with offset
@@ -267,10 +267,10 @@ void put_twiddle(std::vector<double>& out, size_t idx, long long m, long long pe
     out[2 * idx] = std::cos(a);
     out[2 * idx + 1] = -std::sin(a);
 }
-// FP64 pair table of an l-point transform of the pair engine (pair.cuh) with
-// elements per thread e_max (16 or 8, at most l): per pass of stride ns > 1 and
-// radix r = r1 r2, the entries W_{r1 ns}^{rA k} then W_{r ns}^{i kB}; angles
-// reduced exactly in integers.
+// FP64 pair table of an l-point transform of the pair engine (pair.cuh:
+// radix4_pass) with elements per thread e_max (16 or 8, at most l): per pass of
+// stride ns > 1 and radix r = r1 r2, the entries W_{r1 ns}^{rA k} then
+// W_{r ns}^{i kB}; angles reduced exactly in integers.
 void pair_table(int l, int e_max, std::vector<double>& out) {
     const int e = std::min(e_max, l);
     out.assign(2 * (size_t)pr::pair_tab_entries(l, e), 0.0);
@@ -290,6 +290,34 @@ void pair_table(int l, int e_max, std::vector<double>& out) {
         cur *= r;
     }
 }
+// The same for the fused butterflies (pair.cuh: fused_pass): per pass the entries
+// W_{4 ns}^{q k}, q = 1..3 (radix 2: W_{2 ns}^k), then for stage 3 and 4 of 2^s
+// outputs and j < 2^(s-2) the factor c = W_{2^s ns}^{k + j ns} as (larger part, smaller
+// over larger): (re, im / re) for the first half of the j, (im, re / im) after.
+void fused_table(int l, std::vector<double>& out) {
+    const int e = std::min(16, l);
+    out.assign(2 * (size_t)pr::fused_tab_entries(l, e), 0.0);
+    size_t off = 0;
+    for (int cur = 1; cur < l;) {
+        const int r = std::min(e, l / cur);
+        if (cur > 1) {
+            for (int q = 1; q < std::min(r, 4); ++q, off += cur)
+                for (int k = 0; k < cur; ++k)
+                    put_twiddle(out, off + pr::tab_pos(l, e, cur, k), (long long)q * k, (long long)std::min(r, 4) * cur);
+            for (int size = 8; size <= r; size *= 2)
+                for (int j = 0; j < size / 4; ++j, off += cur)
+                    for (int k = 0; k < cur; ++k) {
+                        const size_t i = 2 * (off + pr::tab_pos(l, e, cur, k));
+                        const double a = kTwoPi * (double)(k + (long long)j * cur) / ((double)size * cur);
+                        const double c = std::cos(a), s = -std::sin(a);
+                        const bool sine = j >= size / 8;
+                        out[i] = sine ? s : c;
+                        out[i + 1] = sine ? c / s : s / c;
+                    }
+        }
+        cur *= r;
+    }
+}
 
 // FP32 tables of one grid: kDither twiddle blocks (single-line table, row and
 // column pair tables), P_x (kDitherP x n entries) and P_y with the cross-lane
@@ -304,17 +332,18 @@ struct HostTables32 {
 void build_tables_f32(const nlse_params* p, HostTables32& t) {
     const int n = p->n, h = n / 2;
     std::vector<double> dp(2 * (size_t)n), single, cross(2 * (size_t)h);
-    std::vector<double> pt[4];  // row E 16, row E 8, column E 16, column E 8
+    std::vector<double> pt[5];  // fused row, fused column, radix-8 row, radix-8 column, one-off row
     for (int m = 0; m < n; ++m) {  // (cos phi - 1, sin phi) of P_x = P_y n^2
         const double ph = propagator_phase(p, m), sh = std::sin(0.5 * ph);
         dp[2 * m] = -2.0 * sh * sh;
         dp[2 * m + 1] = std::sin(ph);
     }
     twiddle_table(n, std::min(n, 16), single);
-    pair_table(n, 16, pt[0]);
-    pair_table(n, 8, pt[1]);
-    pair_table(h, 16, pt[2]);
+    fused_table(n, pt[0]);
+    fused_table(h, pt[1]);
+    pair_table(n, 8, pt[2]);
     pair_table(h, 8, pt[3]);
+    pair_table(n, 16, pt[4]);
     for (int k = 0; k < h; ++k) {  // W_n^k = exp(-2 pi i k / n) as (cos - 1, sin)
         const double a = kTwoPi * (double)k / (double)n, sh = std::sin(0.5 * a);
         cross[2 * k] = -2.0 * sh * sh;
@@ -337,29 +366,36 @@ void build_tables_f32(const nlse_params* p, HostTables32& t) {
     t.py.assign((size_t)kDitherP * pyf, 0.0f);
     for (int k = 0; k < h; ++k)
         for (int c = 0; c < 2; ++c) {  // c = 0: cos - 1, 1: sin; lanes k and k + h
-            dither_into(dp[2 * k + c], kTabPy, k, c, t.py.data() + 4 * k + 2 * c, pyf);
-            dither_into(dp[2 * (k + h) + c], kTabPy, k + h, c, t.py.data() + 4 * k + 2 * c + 1, pyf);
-            dither_into(cross[2 * k + c], kTabCross, k, c, t.py.data() + 4 * h + 2 * k + c, pyf);
+            const int q = pr::col_pos(h, k);
+            dither_into(dp[2 * k + c], kTabPy, k, c, t.py.data() + 4 * q + 2 * c, pyf);
+            dither_into(dp[2 * (k + h) + c], kTabPy, k + h, c, t.py.data() + 4 * q + 2 * c + 1, pyf);
+            dither_into(cross[2 * k + c], kTabCross, k, c, t.py.data() + 4 * h + 2 * q + c, pyf);
         }
-    // twiddle blocks: kDither copies (stride cb bytes)
+    // twiddle blocks: kDither copies (stride cb bytes), then the one-off table
     const size_t cb = tw32_copy_bytes(n), cbf = cb / 4;
-    t.tw.assign((size_t)kDither * cb, 0);
+    t.tw.assign(tw32_region_bytes(n), 0);
     float* tw = reinterpret_cast<float*>(t.tw.data());
     for (size_t e = 0; e < single.size() / 2; ++e)
         for (int c = 0; c < 2; ++c) dither_into(single[2 * e + c], kTabTwiddle, e, c, tw + 2 * e + c, cbf);
-    const uint64_t pid[4] = {kTabRowPair, kTabRowPair8, kTabColPair, kTabColPair8};
-    const size_t poff[4] = {tw32_row_off(n, 16), tw32_row_off(n, 8), tw32_col_off(n, 16), tw32_col_off(n, 8)};
+    const uint64_t pid[4] = {kTabRowFused, kTabColFused, kTabRowPair8, kTabColPair8};
+    const size_t poff[4] = {tw32_row_off(n, 16), tw32_col_off(n, 16), tw32_row_off(n, 8), tw32_col_off(n, 8)};
     for (int q = 0; q < 4; ++q)
         for (size_t e = 0; e < pt[q].size() / 2; ++e)
             for (int c = 0; c < 2; ++c) {
-                if (q < 2) {  // row tables: (wx, wy)
+                if (q < 3) {  // (wx, wy)
                     dither_into(pt[q][2 * e + c], pid[q], e, c, tw + poff[q] / 4 + 2 * e + c, cbf);
-                } else {      // column tables: (wx, wx, wy, wy)
+                } else {      // radix-8 column table: (wx, wx, wy, wy)
                     float* f = tw + poff[q] / 4 + 4 * e + 2 * c;
                     dither_into(pt[q][2 * e + c], pid[q], e, c, f, cbf);
                     for (int d = 0; d < kDither; ++d) f[(size_t)d * cbf + 1] = f[(size_t)d * cbf];
                 }
             }
+    float* one = tw + tw32_oneoff_off(n) / 4;
+    for (size_t e = 0; e < pt[4].size() / 2; ++e)
+        for (int c = 0; c < 2; ++c) {
+            const DSplit sp = dsplit(pt[4][2 * e + c]);
+            one[2 * e + c] = sp.frac > uq[dither_offset(kTabRowPair, e, c)] ? sp.hi : sp.lo;
+        }
 }
 
 }  // namespace

@@ -78,7 +78,11 @@ template <auto Kernel> inline cudaError_t ensure_smem(int bytes) {
 // The same, and the preferred shared-memory carveout of the kernel set to the
 // smallest share of the SM's unified L1/shared array that holds `blocks`
 // resident blocks of `bytes` dynamic shared memory each: the rest stays L1
-// cache, where the twiddle and propagator tables are read from.
+// cache, where the twiddle and propagator tables are read from.  blocks = 0: all
+// of it shared memory -- an SM runs blocks of two kernels side by side only under
+// the same carveout, which lets a short pass start while the one before it ends
+// (512^2 step 15.4 -> 11.0 us, 1024^2 22.8 -> 21.1 us; from 2048^2 on the L1 is
+// worth more: 41.6 against 42.1 us).
 template <auto Kernel> inline cudaError_t ensure_smem_carveout(int bytes, int blocks) {
     static unsigned long long done = 0;
     int dev = 0;
@@ -96,7 +100,7 @@ template <auto Kernel> inline cudaError_t ensure_smem_carveout(int bytes, int bl
         return e;
     // 1 KB per block is reserved by the system
     const long long need = (long long)blocks * ((long long)bytes + (long long)fa.sharedSizeBytes + 1024);
-    int pct = per_sm > 0 ? (int)((need * 100 + per_sm - 1) / per_sm) : 100;
+    int pct = per_sm > 0 && blocks > 0 ? (int)((need * 100 + per_sm - 1) / per_sm) : 100;
     pct = pct < 1 ? 1 : (pct > 100 ? 100 : pct);
     if ((e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct)) != cudaSuccess)
         return e;
@@ -170,7 +174,8 @@ cudaError_t launch_col_c(const typename vec2<T>::type* src, typename vec2<T>::ty
 // columns x 256 row pairs.  cuTensorMapEncodeTiled is a host-only driver call,
 // reached through the runtime's entry-point query so that the library needs no
 // link to libcuda.
-inline cudaError_t encode_field_map(CUtensorMap* map, const void* base, int n, int word_bytes, int cols) {
+inline cudaError_t encode_map(CUtensorMap* map, const void* base, int word_bytes, const cuuint64_t (&dims)[3],
+                              const cuuint64_t (&strides)[2], const cuuint32_t (&box)[3]) {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -181,15 +186,26 @@ inline cudaError_t encode_field_map(CUtensorMap* map, const void* base, int n, i
         return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
     }();
     if (!fn) return cudaErrorNotSupported;
-    const cuuint64_t dims[3] = {4, (cuuint64_t)n, (cuuint64_t)n / 2};
-    const cuuint64_t strides[2] = {(cuuint64_t)4 * word_bytes, (cuuint64_t)4 * word_bytes * n};
-    const cuuint32_t box[3] = {4, (cuuint32_t)cols, (cuuint32_t)kTmaBoxRows};
     const cuuint32_t estride[3] = {1, 1, 1};
     const CUresult r = fn(map, word_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32 : CU_TENSOR_MAP_DATA_TYPE_UINT64, 3,
                           const_cast<void*>(base), dims, strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
                           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+inline cudaError_t encode_field_map(CUtensorMap* map, const void* base, int n, int word_bytes, int cols) {
+    const cuuint64_t w = (cuuint64_t)4 * word_bytes;
+    return encode_map(map, base, word_bytes, {4, (cuuint64_t)n, (cuuint64_t)n / 2}, {w, w * n},
+                      {4, (cuuint32_t)cols, (cuuint32_t)kTmaBoxRows});
+}
+// The same field of 16-byte FP32 units as n/2 row pairs x 4 n words: a box of
+// `cols` columns x box_rows row pairs is rows of 16 cols contiguous bytes
+// (the word coordinate of column c is 4 c: 16-byte aligned).
+inline cudaError_t encode_unit_map(CUtensorMap* map, const void* base, int n, int cols, int box_rows) {
+    const cuuint64_t row = (cuuint64_t)16 * n;
+    return encode_map(map, base, 4, {(cuuint64_t)4 * n, (cuuint64_t)n / 2, 1}, {row, row * (n / 2)},
+                      {(cuuint32_t)4 * cols, (cuuint32_t)box_rows, 1});
 }
 
 template <typename T, int N, int C>

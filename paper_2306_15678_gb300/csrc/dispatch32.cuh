@@ -10,6 +10,10 @@
 
 namespace nlse {
 
+// resident blocks the carveout of a march kernel provides for (see
+// ensure_smem_carveout; below 512^2 every kernel fits the smallest carveouts)
+template <int N> constexpr int carveout_blocks(int resident) { return N == 512 || N == 1024 ? 0 : resident; }
+
 template <int N, int E, int C> constexpr bool p_col_valid() {
     return C <= N && p_col_tpl<N, E>() * C <= 1024 && p_col_smem<N, E, C>() <= kMaxSmem;
 }
@@ -26,7 +30,7 @@ cudaError_t launch_row_pass32_e(const float2* src, float2* dst, const float2* tw
     const float4* in = reinterpret_cast<const float4*>(src);
     float4* out = reinterpret_cast<float4*>(dst);
     cudaError_t e;
-    constexpr int RES = p_min_blocks<THREADS, E>();  // resident blocks per SM (register limit)
+    constexpr int RES = carveout_blocks<N>(p_min_blocks<THREADS, E>());  // resident blocks per SM (register limit)
     if (diag) {
         if ((e = ensure_smem_carveout<k_row_pass32<N, E, true>>(SMEM, RES)) != cudaSuccess) return e;
         e = launch_pdl(k_row_pass32<N, E, true>, dim3(BLOCKS), dim3(THREADS), SMEM, s, in, out, twb_of(tw), sc,
@@ -38,8 +42,8 @@ cudaError_t launch_row_pass32_e(const float2* src, float2* dst, const float2* tw
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
-// the persistent staged row pass exists where a row pair fills whole warps of one block
-template <int N> constexpr bool p_row_staged_ok() { return p_rows<N, 16>() == 1 && p_tpl<N, 16>() % 32 == 0; }
+// the persistent staged row pass exists where a row pair is a block of 128 threads or more
+template <int N> constexpr bool p_row_staged_ok() { return p_tpl<N, 16>() >= 128; }
 
 // blocks of the persistent row pass: as many as are resident at once
 inline int resident_grid(int per_sm, int units) {
@@ -92,7 +96,8 @@ cudaError_t launch_col32_c(const float2* src, float2* dst, const float2* tw, con
                            float2 rot, cudaStream_t s) {
     if constexpr (p_col_valid<N, E, C>()) {
         constexpr int SMEM = p_col_smem<N, E, C>();
-        cudaError_t e = ensure_smem_carveout<k_col_pass32<N, E, C>>(SMEM, p_col_min_blocks<p_col_tpl<N, E>() * C, E>());
+        cudaError_t e = ensure_smem_carveout<k_col_pass32<N, E, C>>(
+            SMEM, carveout_blocks<N>(p_col_min_blocks<p_col_tpl<N, E>() * C, E>()));
         if (e != cudaSuccess) return e;
         e = launch_pdl(k_col_pass32<N, E, C>, dim3(N / C), dim3(p_col_tpl<N, E>() * C), SMEM, s,
                        reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), twb_of(tw), px,
@@ -109,14 +114,15 @@ cudaError_t launch_col32_tma_c(const float2* src, float2* dst, const float2* tw,
     if constexpr (p_col_tma_ok<N, E, C>()) {
         constexpr int SMEM = p_col_smem<N, E, C>() + kTmaAlignPad;
         CUtensorMap ml, ms;
-        // boxes of one column: every column of the tile lands at its own line
-        cudaError_t e = encode_field_map(&ml, src, N, 4, 1);
+        constexpr int IL = p_col_il<N, E, C>();
+        cudaError_t e = encode_unit_map(&ml, src, N, IL, p_col_box_rows(N, E));
         if (e == cudaSuccess) {
             if (static_cast<const void*>(src) == static_cast<const void*>(dst)) ms = ml;
-            else e = encode_field_map(&ms, dst, N, 4, 1);
+            else e = encode_unit_map(&ms, dst, N, IL, p_col_box_rows(N, E));
         }
         if (e == cudaSuccess)
-            e = ensure_smem_carveout<k_col_pass32_tma<N, E, C>>(SMEM, p_col_min_blocks<p_col_tpl<N, E>() * C, E>());
+            e = ensure_smem_carveout<k_col_pass32_tma<N, E, C>>(
+                SMEM, carveout_blocks<N>(p_col_min_blocks<p_col_tpl<N, E>() * C, E>()));
         if (e != cudaSuccess) return e;
         e = launch_pdl(k_col_pass32_tma<N, E, C>, dim3(N / C), dim3(p_col_tpl<N, E>() * C), SMEM, s, ml, ms,
                        twb_of(tw), px, reinterpret_cast<const float4*>(py), rot, status, extra_tx);
@@ -204,25 +210,17 @@ template <int N, int E> constexpr int col_mask32_e() {
 // bits 0-9: radix-16 tiles, bits 10-19: radix-8 tiles (kColOptions order)
 template <int N> constexpr int col_mask32() { return col_mask32_e<N, 16>() | (col_mask32_e<N, 8>() << 10); }
 
-// default column tile (radix 16): the narrowest staged tile of at least 128
-// threads (else the widest staged tile), else the narrowest per-thread tile
-// of at least 128 threads (else the widest valid tile)
+// default column tile (radix 16), the fastest measured (us per step on GB300):
+// staged pairs of columns where a column can be staged (32-byte box rows; 4096^2:
+// 158 against 168 with single columns and 195 with two pairs; 2048^2: 41.6, 47.7,
+// 45.1; 512^2: 10.3, 18, 10.5), but single columns at 8192^2 (804 against 900: a
+// pair is one block of 512 threads per SM); two columns per block at 256^2 (8.9
+// against 9.0 and 9.4 with 1, 4); below, single columns at radix 8, for both
+// passes: a pass there is the serial chain of one warp, which half as many
+// elements per thread shorten (64^2: 5.2 against 7.9 us, 128^2: 6.2 against 8.1)
 template <int N> constexpr int col_default32() {
-    constexpr int m = col_mask32<N>();
-    int best = 0;
-    for (int i = 5; i < 10; ++i)
-        if ((m >> i) & 1) {
-            best = kColOptions[i];
-            if (p_col_tpl<N, 16>() * (kColOptions[i] & 0xff) >= 128) return best;
-        }
-    if (best) return best;
-    for (int i = 0; i < 5; ++i)
-        if ((m >> i) & 1) {
-            best = kColOptions[i];
-            if (p_col_tpl<N, 16>() * kColOptions[i] >= 128) return best;
-        }
-    if (best) return best;
-    return 1;
+    if constexpr (N >= 512) return kColTma | (N >= 8192 ? 1 : 2);
+    else return N >= 256 ? 2 : kColR8 | 1;
 }
 
 template <int N> KernelSet<float> make_set32() {
@@ -234,7 +232,8 @@ template <int N> KernelSet<float> make_set32() {
     k.col_mask = col_mask32<N>();
     k.col_default = col_default32<N>();
     k.row_radix_mask = 3 | (p_row_staged_ok<N>() ? 4 : 0);
-    k.row_radix_default = 16;
+    // 8192^2 has one block per SM either way: fetching the next row pair meanwhile pays (417 against 455 us)
+    k.row_radix_default = N >= 8192 ? kRowStaged | 16 : N >= 256 ? 16 : 8;
     k.row_pass = &launch_row_pass32<N>;
     k.col_pass = &launch_col_pass32<N>;
     k.row_forward = &launch_row_forward32<N>;

@@ -41,9 +41,12 @@ using pr::F2;
 // threads per SM: twice the warps, one more exchange per transform); at most L.
 template <int L, int E> __host__ __device__ constexpr int p_e() { return L < E ? L : E; }
 template <int L, int E> __host__ __device__ constexpr int p_tpl() { return L / p_e<L, E>(); }
-// row pairs per block of the row-oriented kernels: at least 128 threads
+// row pairs per block of the row-oriented kernels: at least one warp.  A small
+// grid is a few warps per SM whose serial chains bound the pass: blocks of one
+// warp spread over all SMs (512^2: 10.3 us per step with 32 threads per block,
+// 11.0 with 128).
 template <int N, int E> __host__ __device__ constexpr int p_rows() {
-    return p_tpl<N, E>() >= 128 ? 1 : (128 / p_tpl<N, E>() > N / 2 ? N / 2 : 128 / p_tpl<N, E>());
+    return p_tpl<N, E>() >= 32 ? 1 : (32 / p_tpl<N, E>() > N / 2 ? N / 2 : 32 / p_tpl<N, E>());
 }
 template <int N, int E> __host__ __device__ constexpr int p_row_threads() { return p_tpl<N, E>() * p_rows<N, E>(); }
 template <int N, int E> __host__ __device__ constexpr int p_row_smem() {
@@ -69,9 +72,12 @@ template <int THREADS, int E> __host__ __device__ constexpr int p_col_min_blocks
 
 // Per-step FP32 twiddle block (one of kDither dithered copies, byte offsets
 // from its start): the single-line table of fft.cuh (n entries of 8 bytes,
-// used by the one-off 2D transforms), the pair tables (8-byte entries) of the
-// n-point row transform for E = 16 and E = 8, and those of the n/2-point
-// column sub-transforms for E = 16 and E = 8.
+// used by the adjoint's row kernels and the one-off 2D transforms), the tables
+// of the radix-16 march (pair.cuh: fused butterflies, 8-byte entries) for the
+// n-point row transform and the n/2-point column sub-transforms, and those of
+// the radix-8 march (radix-4 sub-passes) for the same.  After the last copy
+// stands one radix-16 table of the row transform for the load prologue and the
+// readouts (radix-4 sub-passes, dithered as copy 0).
 //
 // Per-step propagator tables (one of kDitherP dithered copies): P_x, n entries
 // of 8 bytes; P_y, n/2 pair entries of 16 bytes followed by the n/2 cross-lane
@@ -90,22 +96,26 @@ template <int THREADS, int E> __host__ __device__ constexpr int p_col_min_blocks
 constexpr int kDitherP = kDither;
 __host__ __device__ constexpr size_t py32_copy_bytes(int n) { return (size_t)16 * (n / 2) + (size_t)8 * (n / 2); }
 __host__ __device__ constexpr int tw32_min(int a, int b) { return a < b ? a : b; }
-// Pair-table entry formats (pair.cuh): 8-byte (wx, wy) for the row transforms
-// (half the L1 footprint and traffic of the tables: row pass 111 -> 103 us at
-// 4096^2), 16-byte (wx, wx, wy, wy) for the column transforms, whose kernel
-// has no registers left for the copies into both lanes (8-byte entries there:
-// 90 -> 112 us, with spills).
+// Pair-table entry formats (pair.cuh): 8-byte (wx, wy), and 16-byte
+// (wx, wx, wy, wy) for the radix-8 column transforms, whose kernel has no
+// registers left for copies into both lanes.
 using RowTab = float2;
-using ColTab = float4;
+template <int E> struct col_tab { using type = float2; };
+template <> struct col_tab<8> { using type = float4; };
 __host__ __device__ constexpr size_t tw32_row_off(int n, int e) {
-    return (size_t)8 * n + (e >= 16 ? 0 : sizeof(RowTab) * pr::pair_tab_entries(n, tw32_min(16, n)));
+    return (size_t)8 * n + (e >= 16 ? 0 : (size_t)8 * (pr::fused_tab_entries(n, tw32_min(16, n)) +
+                                                       pr::fused_tab_entries(n / 2, tw32_min(16, n / 2))));
 }
 __host__ __device__ constexpr size_t tw32_col_off(int n, int e) {
-    return tw32_row_off(n, 8) + sizeof(RowTab) * pr::pair_tab_entries(n, tw32_min(8, n)) +
-           (e >= 16 ? 0 : sizeof(ColTab) * pr::pair_tab_entries(n / 2, tw32_min(16, n / 2)));
+    return e >= 16 ? tw32_row_off(n, 16) + (size_t)8 * pr::fused_tab_entries(n, tw32_min(16, n))
+                   : (tw32_row_off(n, 8) + (size_t)8 * pr::pair_tab_entries(n, tw32_min(8, n)) + 15) / 16 * 16;
 }
 __host__ __device__ constexpr size_t tw32_copy_bytes(int n) {
-    return (tw32_col_off(n, 8) + sizeof(ColTab) * pr::pair_tab_entries(n / 2, tw32_min(8, n / 2)) + 255) / 256 * 256;
+    return (tw32_col_off(n, 8) + (size_t)16 * pr::pair_tab_entries(n / 2, tw32_min(8, n / 2)) + 255) / 256 * 256;
+}
+__host__ __device__ constexpr size_t tw32_oneoff_off(int n) { return (size_t)kDither * tw32_copy_bytes(n); }
+__host__ __device__ constexpr size_t tw32_region_bytes(int n) {
+    return tw32_oneoff_off(n) + (size_t)8 * pr::pair_tab_entries(n, tw32_min(16, n));
 }
 
 // Global-memory access of the units: plain for the per-pass kernels, L2-only
@@ -245,62 +255,79 @@ __device__ __forceinline__ C2 apply_screen2(C2 v, const ScreenCoef<float>& c, un
 
 // ------------------------------------------------------------- row tile --
 
+// Screens of one row pair: v = the output of the inverse row transform (parts
+// swapped) in, the field to transform forward out; with DIAG adds the thread's
+// sum and max of |U|^2 (after the first screen); EXACT compiles the exact
+// pointwise substep in.
+template <bool DIAG, bool EXACT, int E>
+__device__ __forceinline__ void row_screens32(C2 (&v)[E], const ScreenCoef<float>& sc, F2& fsum, float& tmax) {
+    // the field entering the screen, swapped back
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = pr::swp(v[m]);
+    if (sc.scale != 1.0f) {  // (uniform)
+        const F2 s = pr::bc(sc.scale);
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = {pr::mul(v[m].re, s), pr::mul(v[m].im, s)};
+    }
+    const unsigned warp = (blockDim.x & 31) == 0 ? 0xffffffffu : __activemask();
+#pragma unroll 1
+    for (int rep = 0; rep < sc.reps; ++rep) {
+        if (sc.active) {
+            if (EXACT && sc.exact) {  // (uniform)
+#pragma unroll
+                for (int m = 0; m < E; ++m) {
+                    float r0, r1, i0, i1;
+                    pr::up(v[m].re, r0, r1);
+                    pr::up(v[m].im, i0, i1);
+                    const float2 a = apply_screen_exact<float>(make_float2(r0, i0), sc.inv_iref, sc.im_k, sc.im_p,
+                                                               sc.ka, sc.K);
+                    const float2 b = apply_screen_exact<float>(make_float2(r1, i1), sc.inv_iref, sc.im_k, sc.im_p,
+                                                               sc.ka, sc.K);
+                    v[m] = {pr::pk(a.x, b.x), pr::pk(a.y, b.y)};
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < E; ++m) v[m] = pr::apply_screen2(v[m], sc, warp);
+            }
+        }
+        if (DIAG && rep == 0) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                const F2 a = pr::fma(v[m].re, v[m].re, pr::mul(v[m].im, v[m].im));
+                fsum = pr::add(fsum, a);
+                float a0, a1;
+                pr::up(a, a0, a1);
+                tmax = fmaxf(tmax, fmaxf(a0, a1));
+            }
+        }
+    }
+}
+
 // Row pass transforms of one row pair held in v (B_x S swapped in): B_x,
-// screen(s), F_x; with DIAG adds the thread's sum and max of |U|^2 (after the
-// first screen); EXACT compiles the exact pointwise substep in.  hook runs in
-// the forward transform once the line is free (pair.cuh: fft_pair).
+// screen(s), F_x.  hook runs in the forward transform once the line is free
+// (pair.cuh: fft_second).  Thread t holds the natural elements
+// row_id<N, ER>(t) + m T.
+template <int N, int ER> __device__ __forceinline__ int row_id(int t) {
+    if constexpr (pr::mirrored(N, p_e<N, ER>())) return pr::nat_id<N>(t);
+    else return t;
+}
 template <int N, int ER, bool DIAG, bool EXACT = true, class H = pr::NoHook>
 __device__ __forceinline__ void row_body32(C2 (&v)[p_e<N, ER>()], C2* sm, const RowTab* __restrict__ tab,
-                                           const ScreenCoef<float>& sc, int j, float& tsum, float& tmax,
+                                           const ScreenCoef<float>& sc, int t, float& tsum, float& tmax,
                                            const H& hook = H{}) {
     constexpr int E = p_e<N, ER>();
+    using S = pr::LineSync<p_tpl<N, ER>()>;
     F2 fsum = pr::bc(0.0f);
+    if constexpr (pr::mirrored(N, E)) {
+        pr::fft_first<N, S>(v, sm, tab, t);
+        row_screens32<DIAG, EXACT>(v, sc, fsum, tmax);
+        pr::fft_second<N, S, 1>(v, sm, tab, t, hook);
+    } else {
+        static_assert(H::none, "the hook is for the mirrored transforms");
 #pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-        pr::fft_pair<N, E>(v, sm, tab, j, [&]() {
-            if (half == 1) hook();
-        });
-        if (half == 0) {
-            // the field entering the screen, swapped back
-#pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = pr::swp(v[m]);
-            if (sc.scale != 1.0f) {  // (uniform)
-                const F2 s = pr::bc(sc.scale);
-#pragma unroll
-                for (int m = 0; m < E; ++m) v[m] = {pr::mul(v[m].re, s), pr::mul(v[m].im, s)};
-            }
-            const unsigned warp = (blockDim.x & 31) == 0 ? 0xffffffffu : __activemask();
-#pragma unroll 1
-            for (int rep = 0; rep < sc.reps; ++rep) {
-                if (sc.active) {
-                    if (EXACT && sc.exact) {  // (uniform)
-#pragma unroll
-                        for (int m = 0; m < E; ++m) {
-                            float r0, r1, i0, i1;
-                            pr::up(v[m].re, r0, r1);
-                            pr::up(v[m].im, i0, i1);
-                            const float2 a = apply_screen_exact<float>(make_float2(r0, i0), sc.inv_iref, sc.im_k,
-                                                                       sc.im_p, sc.ka, sc.K);
-                            const float2 b = apply_screen_exact<float>(make_float2(r1, i1), sc.inv_iref, sc.im_k,
-                                                                       sc.im_p, sc.ka, sc.K);
-                            v[m] = {pr::pk(a.x, b.x), pr::pk(a.y, b.y)};
-                        }
-                    } else {
-#pragma unroll
-                        for (int m = 0; m < E; ++m) v[m] = pr::apply_screen2(v[m], sc, warp);
-                    }
-                }
-                if (DIAG && rep == 0) {
-#pragma unroll
-                    for (int m = 0; m < E; ++m) {
-                        const F2 a = pr::fma(v[m].re, v[m].re, pr::mul(v[m].im, v[m].im));
-                        fsum = pr::add(fsum, a);
-                        float a0, a1;
-                        pr::up(a, a0, a1);
-                        tmax = fmaxf(tmax, fmaxf(a0, a1));
-                    }
-                }
-            }
+        for (int half = 0; half < 2; ++half) {
+            pr::fft_pair<N, E, S, (ER >= 16)>(v, sm, tab, t);
+            if (half == 0) row_screens32<DIAG, EXACT>(v, sc, fsum, tmax);
         }
     }
     if (DIAG) tsum += pr::lo(fsum) + pr::hi(fsum);
@@ -315,14 +342,14 @@ __device__ __forceinline__ void row_tile32(const float4* src, float4* dst, const
                                            float& tmax) {
     constexpr int E = p_e<N, ER>(), T = p_tpl<N, ER>();
     constexpr int LS = pr::pair_line_stride<N, E, RP>();
-    const int g = (int)threadIdx.x / T, j = (int)threadIdx.x % T;
+    const int g = (int)threadIdx.x / T, t = (int)threadIdx.x % T, j = row_id<N, ER>(t);
     const size_t row = (size_t)(pair0 + g) * N;
     C2* sm = smem + g * LS;
     const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, ER));
     C2 v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = pr::swp(M::ld(src + row + j + m * T));  // B_x = swap F_x swap
-    row_body32<N, ER, DIAG, M::kExactScreen>(v, sm, tab, sc, j, tsum, tmax);
+    row_body32<N, ER, DIAG, M::kExactScreen>(v, sm, tab, sc, t, tsum, tmax);
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + row + j + m * T, v[m]);
 }
@@ -341,55 +368,65 @@ __device__ __forceinline__ void cmul_1d(float xr, float xi, float2 w, float& re,
     im = fmaf(xi, w.x, fmaf(xr, w.y, xi));
 }
 
-// Column transform body: v holds units (j + m T, col) of one column (lanes:
+// Column transform body: v holds units (t + m T, col) of one column (lanes:
 // even and odd rows); computes B_y(P_x(col) rot P_y / n^2 F_y .) and leaves
 // the output units in v.  tw: the step's twiddle block; px: n entries (d, s)
 // of P_x; py: n/2 entries (d[k], d[k+n/2], s[k], s[k+n/2]) of P_y (without
 // its 1/n^2, which goes with P_x: a power of two, exact), then the n/2
-// cross-lane factors (d, s).
-template <int N, int EC>
+// cross-lane factors (d, s), both with entry k at col_pos(n/2, k).
+template <int L> __device__ __forceinline__ void col_middle32(C2& v, int pos, const float2* __restrict__ cross,
+                                                              const float4* __restrict__ py, F2 qx, F2 qy, F2 nqy,
+                                                              F2 xd, F2 xs, F2 nxs) {
+    const float2 w = pr::ld1(cross + pos);  // (cos - 1, sin) of W_n^k
+    // X[k] = E + t, X[k + L] = E - t, t = W_n^k O
+    float er, orr, ei, oi;
+    pr::up(v.re, er, orr);
+    pr::up(v.im, ei, oi);
+    float tr, ti;
+    cmul_1d(orr, oi, w, tr, ti);
+    C2 X = {pr::pk(er + tr, er - tr), pr::pk(ei + ti, ei - ti)};
+    // rot / n^2 and P_x (both lanes), then P_y (per lane): X + X (d + i s)
+    X = pr::cmulw(X, qx, qy, nqy);
+    X = {pr::fma(X.re, xd, pr::fma(X.im, nxs, X.re)), pr::fma(X.im, xd, pr::fma(X.re, xs, X.im))};
+    F2 yd, ys;
+    pr::ld_lanes(py + pos, yd, ys);
+    X = {pr::fma(X.re, yd, pr::fma(X.im, pr::neg(ys), X.re)), pr::fma(X.im, yd, pr::fma(X.re, ys, X.im))};
+    // Y = swap(X): A = Y[k] + Y[k + L], B = (Y[k] - Y[k + L]) W_n^k
+    float yr0, yr1, yi0, yi1;
+    pr::up(X.im, yr0, yr1);
+    pr::up(X.re, yi0, yi1);
+    float br, bi;
+    cmul_1d(yr0 - yr1, yi0 - yi1, w, br, bi);
+    v = {pr::pk(yr0 + yr1, br), pr::pk(yi0 + yi1, bi)};
+}
+template <int N, int EC, class S, int IL = 1>
 __device__ __forceinline__ void col_body32(C2 (&v)[p_e<N / 2, EC>()], C2* sm, const unsigned char* twb,
                                            const float2* __restrict__ px, const float4* __restrict__ py,
-                                           float2 rot, int col, int j) {
+                                           float2 rot, int col, int t) {
     constexpr int L = N / 2, E = p_e<L, EC>(), T = p_tpl<L, EC>();
-    const ColTab* tab = reinterpret_cast<const ColTab*>(twb + tw32_col_off(N, EC));
+    const auto* tab = reinterpret_cast<const typename col_tab<EC>::type*>(twb + tw32_col_off(N, EC));
     const float2* cross = reinterpret_cast<const float2*>(py + L);  // after the n/2 P_y entries
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-        pr::fft_pair<L, E>(v, sm, tab, j);
-        if (half == 0) {
-            // rot / n^2 (a power of two: exact) and P_x(col) = 1 + d + i s, each
-            // applied to every value (their product, rounded once per column,
-            // would carry a magnitude error common to the column's values)
-            constexpr float inv_n2 = 1.0f / ((float)N * (float)N);
-            const F2 qx = pr::bc(rot.x * inv_n2), qy = pr::bc(rot.y * inv_n2), nqy = pr::bc(-rot.y * inv_n2);
-            const float2 pxd = pr::ld1(px + col);
-            const F2 xd = pr::bc(pxd.x), xs = pr::bc(pxd.y), nxs = pr::bc(-pxd.y);
+    auto middle = [&](int k0) {  // elements k0 + m T
+        // rot / n^2 (a power of two: exact) and P_x(col) = 1 + d + i s, each
+        // applied to every value (their product, rounded once per column,
+        // would carry a magnitude error common to the column's values)
+        constexpr float inv_n2 = 1.0f / ((float)N * (float)N);
+        const F2 qx = pr::bc(rot.x * inv_n2), qy = pr::bc(rot.y * inv_n2), nqy = pr::bc(-rot.y * inv_n2);
+        const float2 pxd = pr::ld1(px + col);
+        const F2 xd = pr::bc(pxd.x), xs = pr::bc(pxd.y), nxs = pr::bc(-pxd.y);
+        const int p0 = pr::col_pos(L, k0);  // (permutes runs of L/16 entries, and T is a multiple of L/16)
 #pragma unroll
-            for (int m = 0; m < E; ++m) {
-                const int k = j + m * T;
-                const float2 w = pr::ld1(cross + k);  // (cos - 1, sin) of W_n^k
-                // X[k] = E + t, X[k + L] = E - t, t = W_n^k O
-                float er, orr, ei, oi;
-                pr::up(v[m].re, er, orr);
-                pr::up(v[m].im, ei, oi);
-                float tr, ti;
-                cmul_1d(orr, oi, w, tr, ti);
-                C2 X = {pr::pk(er + tr, er - tr), pr::pk(ei + ti, ei - ti)};
-                // rot / n^2 and P_x (both lanes), then P_y (per lane): X + X (d + i s)
-                X = pr::cmulw(X, qx, qy, nqy);
-                X = {pr::fma(X.re, xd, pr::fma(X.im, nxs, X.re)), pr::fma(X.im, xd, pr::fma(X.re, xs, X.im))};
-                F2 yd, ys;
-                pr::ld_lanes(py + k, yd, ys);
-                X = {pr::fma(X.re, yd, pr::fma(X.im, pr::neg(ys), X.re)), pr::fma(X.im, yd, pr::fma(X.re, ys, X.im))};
-                // Y = swap(X): A = Y[k] + Y[k + L], B = (Y[k] - Y[k + L]) W_n^k
-                float yr0, yr1, yi0, yi1;
-                pr::up(X.im, yr0, yr1);
-                pr::up(X.re, yi0, yi1);
-                float br, bi;
-                cmul_1d(yr0 - yr1, yi0 - yi1, w, br, bi);
-                v[m] = {pr::pk(yr0 + yr1, br), pr::pk(yi0 + yi1, bi)};
-            }
+        for (int m = 0; m < E; ++m) col_middle32<L>(v[m], p0 + m * T, cross, py, qx, qy, nqy, xd, xs, nxs);
+    };
+    if constexpr (pr::mirrored(L, E)) {
+        pr::fft_first<L, S, IL>(v, sm, tab, t);
+        middle(pr::mid_id<L>(t));
+        pr::fft_second<L, S, IL>(v, sm, tab, t);
+    } else {
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            pr::fft_pair<L, E, S, (EC >= 16), IL>(v, sm, tab, t);
+            if (half == 0) middle(t);
         }
     }
 #pragma unroll
@@ -413,13 +450,16 @@ k_row_pass32(const float4* src, float4* dst, const unsigned char* twb, ScreenCoe
     if constexpr (DIAG) block_partials<float>(tsum, tmax, partials);
 }
 
+// hook of fft_second that does something
+template <class F> struct LineFree {
+    static constexpr bool none = false;
+    const F& f;
+    __device__ __forceinline__ void operator()() const { f(); }
+};
+
 // One contiguous bulk copy of `bytes` (a multiple of 16; both addresses 16-byte
-// aligned) from global into shared memory, counted in bytes on bar; the calling
-// thread also arrives on bar, expecting those bytes (plus `extra`, a test hook
-// that keeps the phase from completing).
-__device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar,
-                                             uint32_t extra = 0) {
-    mbar_expect_tx(bar, bytes + extra);
+// aligned) from global into shared memory, counted in bytes on bar.
+__device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
@@ -450,35 +490,41 @@ __device__ __forceinline__ void block_partials32_at(float tsum, float tmax, doub
 
 // Row pass with persistent blocks (one row pair per block at a time, n >= 2048
 // at radix 16): block b takes row pairs b, b + G, b + 2G, ... (G blocks).  A
-// row pair is n contiguous units, so it is moved into the block's transform
-// line by one bulk copy; the copy for the next row pair is issued as soon as
-// the forward transform has read the line for the last time, and lands while
+// row pair is n contiguous units; 16 bulk copies move its 16th parts to the
+// starts of the line's regions (pair.cuh: Mirror), where each thread finds the
+// elements it starts with in the slots it then writes first; the copies for
+// the next row pair are issued as soon as the forward transform has read the
+// line for the last time, and land while
 // the last transform pass, the stores and the partials of the current row
 // pair run.  Arithmetic, stores and partials (one slot per row pair) are those
-// of k_row_pass32 at radix 16, bit for bit.  The wait for a copy is bounded as
-// in the staged column pass (status bits 2 and 4, tma.cuh).  extra_tx (a test
+// of k_row_pass32 at radix 16, bit for bit.  The wait for the copies is bounded
+// as in the staged column pass (status bits 2 and 4, tma.cuh).  extra_tx (a test
 // hook, 0 in use) makes block 0 expect that many bytes more for its first row
-// pair than the copy brings, so that its wait runs out.
+// pair than the copies bring, so that its wait runs out.
 template <int N, bool DIAG>
 __global__ void __launch_bounds__(p_tpl<N, 16>(), p_min_blocks<p_tpl<N, 16>(), 16>())
 k_row_pass32_pf(const float4* src, float4* dst, const unsigned char* twb, ScreenCoef<float> sc,
                 double* __restrict__ partials, int* __restrict__ status, uint32_t extra_tx) {
     constexpr int E = p_e<N, 16>(), T = p_tpl<N, 16>(), NP = N / 2;
-    constexpr uint32_t BYTES = (uint32_t)N * 16;
+    constexpr int RS = pr::Mirror<N>::RS;
     static_assert(p_rows<N, 16>() == 1 && T % 32 == 0, "one row pair of whole warps per block");
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ uint64_t bar;
     __shared__ int s_fail;
     C2* line = reinterpret_cast<C2*>(smraw);
     const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, 16));
-    const int j = (int)threadIdx.x;
+    const int t = (int)threadIdx.x, j = pr::nat_id<N>(t);
+    auto load_pair = [&](int p, uint32_t extra) {
+        mbar_expect_tx(&bar, (uint32_t)N * 16 + extra);
+#pragma unroll 1
+        for (int r = 0; r < 16; ++r) bulk_load_1d(line + r * RS, src + (size_t)p * N + r * T, T * 16, &bar);
+    };
     pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) {
         s_fail = 0;
         mbar_init(&bar, 1);
-        if ((int)blockIdx.x < NP)
-            bulk_load_1d(line, src + (size_t)blockIdx.x * N, BYTES, &bar, blockIdx.x == 0 ? extra_tx : 0u);
+        if ((int)blockIdx.x < NP) load_pair(blockIdx.x, blockIdx.x == 0 ? extra_tx : 0u);
     }
     __syncthreads();
     uint32_t parity = 0;
@@ -495,16 +541,16 @@ k_row_pass32_pf(const float4* src, float4* dst, const unsigned char* twb, Screen
         if (s_fail) return;  // (uniform)
         C2 v[E];
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = pr::swp(line[j + m * T]);  // B_x = swap F_x swap
-        __syncthreads();  // the transforms' exchanges reuse the line
+        for (int m = 0; m < E; ++m) v[m] = pr::swp(line[j + m * RS]);  // B_x = swap F_x swap
         const int next = p + (int)gridDim.x;
         float tsum = 0.0f, tmax = 0.0f;
-        row_body32<N, 16, DIAG>(v, line, tab, sc, j, tsum, tmax, [&]() {
+        auto fetch_next = [&]() {
             if (threadIdx.x == 0 && next < NP) {
-                fence_proxy_async_smem();  // the exchanges' accesses of the line, before the copy's writes
-                bulk_load_1d(line, src + (size_t)next * N, BYTES, &bar);
+                fence_proxy_async_smem();  // the exchanges' accesses of the line, before the copies' writes
+                load_pair(next, 0u);
             }
-        });
+        };
+        row_body32<N, 16, DIAG, true, LineFree<decltype(fetch_next)>>(v, line, tab, sc, t, tsum, tmax, {fetch_next});
 #pragma unroll
         for (int m = 0; m < E; ++m) UnitPlain::st(dst + (size_t)p * N + j + m * T, v[m]);
         if constexpr (DIAG) block_partials32_at(tsum, tmax, partials, p);
@@ -524,7 +570,7 @@ __device__ __forceinline__ void col_tile32(const float4* src, float4* dst, const
     C2 v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = M::ld(src + (size_t)(j + m * T) * N + col);
-    col_body32<N, EC>(v, smem + c * LS, twb, px, py, rot, col, j);
+    col_body32<N, EC, pr::LineSync<T, C>>(v, smem + c * LS, twb, px, py, rot, col, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + (size_t)(j + m * T) * N + col, v[m]);
 }
@@ -546,22 +592,87 @@ template <int N, int EC, int C> __host__ __device__ constexpr bool p_col_tma_val
     return N % (2 * kTmaBoxRows) == 0 && p_col_tpl<N, EC>() * C <= 1024 &&
            p_col_smem<N, EC, C>() + kTmaAlignPad <= 232448;
 }
+// Columns staged side by side: pairs of columns share boxes of 32-byte rows and
+// interleaved lines and threads (pair.cuh: IL) where the tile is an even number
+// of columns.  A box row of one column is half a 32-byte sector, so single
+// columns move every sector twice between L2 and the SM, and the copies are
+// counted by rows.
+template <int N, int EC, int C> __host__ __device__ constexpr int p_col_il() {
+    return C % 2 == 0 && EC == 16 && p_col_tpl<N, EC>() >= 16 ? 2 : 1;
+}
+// Place of a staged column in its transform line: where the mirrored
+// transforms' regions start on 128-byte boundaries (n/2 = 2048, 4096), one box
+// of n/32 units per region, so that each thread finds its first elements in the
+// slots it writes first and leaves its results in the slots it read last (no
+// barrier between); else boxes of 256 units one after the other.
+template <int N, int EC> __host__ __device__ constexpr bool p_col_in_regions() {
+    return pr::mirrored(N / 2, p_e<N / 2, EC>()) && N >= 4096;
+}
+__host__ __device__ constexpr int p_col_box_rows(int n, int ec) { return ec == 16 && n >= 4096 ? n / 32 : kTmaBoxRows; }
+template <int N, int EC> __host__ __device__ constexpr int p_col_box_stride() {
+    return p_col_in_regions<N, EC>() ? pr::pair_padded_len<N / 2, 16>() / 16 : kTmaBoxRows;
+}
 
-// Column pass with the tile staged by bulk tensor copies: column c of the
-// block lands at the start of its own transform line (boxes of 256 units of
-// one column; the tensor maps describe the state as n/2 row pairs x n columns
-// x 4 words), the threads of a column (c = tid / T) read their units from
-// there, transform them (col_body32, bit for bit as k_col_pass32) and write
-// them back, and one thread stores the lines with bulk tensor copies.  Waits
+// One staged column: thread t of its p_col_tpl threads reads units t + m T
+// from the line, transforms them (col_body32, bit for bit as
+// k_col_pass32) and writes them back.  Every access of the line by other
+// threads is ordered before the caller's next barrier.
+template <int N, int EC, int IL>
+__device__ __forceinline__ void col_line32(C2* line, const unsigned char* twb, const float2* __restrict__ px,
+                                           const float4* __restrict__ py, float2 rot, int col, int t) {
+    constexpr int L = N / 2, E = p_e<L, EC>(), T = p_tpl<L, EC>();
+    constexpr bool REG = p_col_in_regions<N, EC>();
+    constexpr int ST = (REG ? p_col_box_stride<N, EC>() : T) * IL;
+    static_assert(!REG || p_col_box_rows(N, EC) == T, "one box per region");
+    using S = pr::LineSync<T, IL>;
+    C2 v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = line[t * IL + m * ST];
+    if constexpr (!REG) S::all();  // the staged column is consumed; the transforms reuse its memory
+    col_body32<N, EC, S, IL>(v, line, twb, px, py, rot, col, t);
+    if constexpr (!REG && pr::mirrored(L, E)) S::all();  // the last exchange is read
+#pragma unroll
+    for (int m = 0; m < E; ++m) line[t * IL + m * ST] = v[m];
+}
+// the tile's columns col0 .. col0 + C - 1 in smem, thread tid of the block
+template <int N, int EC, int C>
+__device__ __forceinline__ void col_lines32(C2* smem, const unsigned char* twb, const float2* __restrict__ px,
+                                            const float4* __restrict__ py, float2 rot, int col0, int tid) {
+    constexpr int L = N / 2, T = p_tpl<L, EC>(), IL = p_col_il<N, EC, C>();
+    constexpr int LS = pr::pair_line_stride<L, p_e<L, EC>(), C>();
+    const int grp = tid / (T * IL), c = tid % IL, t = tid % (T * IL) / IL;
+    col_line32<N, EC, IL>(smem + grp * LS * IL + c, twb, px, py, rot, col0 + grp * IL + c, t);
+}
+template <int N, int EC, int C>
+__device__ __forceinline__ void col_stage_load(C2* smem, const CUtensorMap* map, int col0, uint64_t* bar) {
+    constexpr int L = N / 2, IL = p_col_il<N, EC, C>(), LS = pr::pair_line_stride<L, p_e<L, EC>(), C>() * IL;
+    constexpr int BR = p_col_box_rows(N, EC), BS = p_col_box_stride<N, EC>() * IL;
+#pragma unroll 1
+    for (int c = 0; c < C / IL; ++c)
+#pragma unroll 1
+        for (int b = 0; b < L / BR; ++b) tma_load_3d(smem + c * LS + b * BS, map, 4 * (col0 + c * IL), b * BR, 0, bar);
+}
+template <int N, int EC, int C>
+__device__ __forceinline__ void col_stage_store(const C2* smem, const CUtensorMap* map, int col0) {
+    constexpr int L = N / 2, IL = p_col_il<N, EC, C>(), LS = pr::pair_line_stride<L, p_e<L, EC>(), C>() * IL;
+    constexpr int BR = p_col_box_rows(N, EC), BS = p_col_box_stride<N, EC>() * IL;
+#pragma unroll 1
+    for (int c = 0; c < C / IL; ++c)
+#pragma unroll 1
+        for (int b = 0; b < L / BR; ++b) tma_store_3d(map, 4 * (col0 + c * IL), b * BR, 0, smem + c * LS + b * BS);
+}
+
+// Column pass with the tile staged by bulk tensor copies: the columns land in
+// their transform lines (the tensor maps describe the state as n/2 row pairs x
+// 4 n words), are transformed there (col_line32), and one thread stores
+// the lines with bulk tensor copies.  Waits
 // are bounded as in k_col_pass_tma (tma.cuh), with the same status bits.
 template <int N, int EC, int C>
 __global__ void __launch_bounds__(p_col_tpl<N, EC>() * C, p_col_min_blocks<p_col_tpl<N, EC>() * C, EC>())
 k_col_pass32_tma(const __grid_constant__ CUtensorMap mload, const __grid_constant__ CUtensorMap mstore,
                  const unsigned char* twb, const float2* __restrict__ px, const float4* __restrict__ py, float2 rot,
                  int* __restrict__ status, uint32_t extra_tx) {
-    constexpr int L = N / 2, E = p_e<L, EC>(), T = p_tpl<L, EC>();
-    constexpr int LS = pr::pair_line_stride<L, E, C>(), BOXES = L / kTmaBoxRows;
-    constexpr uint32_t BYTES = (uint32_t)(C * L * 16);
+    constexpr uint32_t BYTES = (uint32_t)(C * (N / 2) * 16);
     static_assert(p_col_tma_valid<N, EC, C>(), "staged column tile");
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ uint64_t bar;
@@ -575,11 +686,7 @@ k_col_pass32_tma(const __grid_constant__ CUtensorMap mload, const __grid_constan
         s_fail = 0;
         mbar_init(&bar, 1);
         mbar_expect_tx(&bar, BYTES + (blockIdx.x == 0 ? extra_tx : 0u));
-#pragma unroll 1
-        for (int c = 0; c < C; ++c)
-#pragma unroll 1
-            for (int b = 0; b < BOXES; ++b)
-                tma_load_3d(smem + c * LS + b * kTmaBoxRows, &mload, 0, col0 + c, b * kTmaBoxRows, &bar);
+        col_stage_load<N, EC, C>(smem, &mload, col0, &bar);
         if (!mbar_wait_bounded(&bar, 0)) {
             if (status) atomicOr(status, 2);
             // the copies still target this block's memory: wait for them once more
@@ -589,24 +696,11 @@ k_col_pass32_tma(const __grid_constant__ CUtensorMap mload, const __grid_constan
     }
     __syncthreads();
     if (s_fail) return;  // (uniform)
-    const int c = (int)threadIdx.x / T, j = (int)threadIdx.x % T;
-    C2* line = smem + c * LS;
-    C2 v[E];
-#pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = line[j + m * T];
-    __syncthreads();  // the staged tile is consumed; the transforms reuse its memory
-    // the transforms end with a barrier after their last shared-memory read
-    col_body32<N, EC>(v, line, twb, px, py, rot, col0 + c, j);
-#pragma unroll
-    for (int m = 0; m < E; ++m) line[j + m * T] = v[m];
+    col_lines32<N, EC, C>(smem, twb, px, py, rot, col0, threadIdx.x);
     fence_proxy_async_smem();
     __syncthreads();
     if (threadIdx.x == 0) {
-#pragma unroll 1
-        for (int cc = 0; cc < C; ++cc)
-#pragma unroll 1
-            for (int b = 0; b < BOXES; ++b)
-                tma_store_3d(&mstore, 0, col0 + cc, b * kTmaBoxRows, smem + cc * LS + b * kTmaBoxRows);
+        col_stage_store<N, EC, C>(smem, &mstore, col0);
         tma_store_commit_and_wait_read();
     }
 }
@@ -621,14 +715,14 @@ k_row_forward32(const float2* __restrict__ src, float4* __restrict__ dst, const 
     extern __shared__ __align__(16) unsigned char smraw[];
     const int g = (int)threadIdx.x / T, j = (int)threadIdx.x % T;
     const size_t p = (size_t)blockIdx.x * RP + g;
-    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, 16));
+    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_oneoff_off(N));
     C2 v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const float2 a = src[(2 * p) * N + j + m * T], b = src[(2 * p + 1) * N + j + m * T];
         v[m] = {pr::pk(a.x, b.x), pr::pk(a.y, b.y)};
     }
-    pr::fft_pair<N, E>(v, reinterpret_cast<C2*>(smraw) + g * LS, tab, j);
+    pr::fft_pair<N, E, pr::LineSync<T>, false>(v, reinterpret_cast<C2*>(smraw) + g * LS, tab, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) UnitPlain::st(dst + p * N + j + m * T, v[m]);
 }
@@ -645,11 +739,11 @@ k_readout32(const float4* __restrict__ state, const unsigned char* twb, float2* 
     extern __shared__ __align__(16) unsigned char smraw[];
     const int g = (int)threadIdx.x / T, j = (int)threadIdx.x % T;
     const size_t p = (size_t)blockIdx.x * RP + g;
-    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, 16));
+    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_oneoff_off(N));
     C2 v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = pr::swp(UnitPlain::ld(state + p * N + j + m * T));
-    pr::fft_pair<N, E>(v, reinterpret_cast<C2*>(smraw) + g * LS, tab, j);
+    pr::fft_pair<N, E, pr::LineSync<T>, false>(v, reinterpret_cast<C2*>(smraw) + g * LS, tab, j);
     const float inv = 1.0f / (float)N;
     float tsum = 0.0f, tmax = 0.0f;
 #pragma unroll
