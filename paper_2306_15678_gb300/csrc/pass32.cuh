@@ -251,6 +251,63 @@ __device__ __forceinline__ C2 apply_screen2(C2 v, const ScreenCoef<float>& c, un
     return {add(v.re, ddx), add(v.im, ddy)};
 }
 
+// The screen of all of a thread's values for K = 8 and real gains (the nominal
+// case).  The largest intensity of the warp's values bounds every phase and gain,
+// so one vote picks the polynomials for all of them and the values follow each
+// other without branches (a vote and two branches per value kept the sixteen
+// dependent chains from overlapping).  Short form: phases within 1/32 rad and
+// gains below 2^-9 (expm1 to x^3, relative truncation below 4e-10; sin to x^5,
+// cos - 1 to x^6, below 1e-13); middle form: phases within pi/4, gains below
+// 1/16; beyond, value by value (apply_screen2).
+template <int FORM> __device__ __forceinline__ C2 screen_k8(C2 v, F2 u, const ScreenCoef<float>& c) {
+    const F2 u2 = mul(u, u), u4 = mul(u2, u2);
+    const F2 re = mul(bc(c.re_a), mul(mul(u4, u2), u));
+    const F2 im = fma(bc(c.im_k), u, mul(bc(c.im_p), mul(u4, u4)));
+    F2 em1, sn, cm1;
+    if constexpr (FORM == 0) {
+        em1 = fma(mul(re, re), fma(re, bc(1.66666666666666667e-1f), bc(0.5f)), re);
+        sin_cosm1_short2(im, sn, cm1);
+    } else {
+        em1 = expm1_core2(re);
+        sin_cosm1_core2(im, sn, cm1);
+    }
+    const F2 dre = fma(em1, cm1, add(em1, cm1));  // (1 + em1)(1 + cm1) - 1
+    const F2 dim = fma(em1, sn, sn);              // (1 + em1) sin
+    const F2 ddx = fma(v.re, dre, mul(v.im, neg(dim)));
+    const F2 ddy = fma(v.re, dim, mul(v.im, dre));
+    return {add(v.re, ddx), add(v.im, ddy)};
+}
+__device__ __forceinline__ F2 screen_u(C2 v, const ScreenCoef<float>& c) {
+    return mul(fma(v.re, v.re, mul(v.im, v.im)), bc(c.inv_iref));
+}
+template <int E> __device__ __forceinline__ void apply_screens2(C2 (&v)[E], const ScreenCoef<float>& c, unsigned warp) {
+    if (c.K == 8 && c.real_gains) {  // (uniform)
+        float um = 0.0f;
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            float u0, u1;
+            up(screen_u(v[m], c), u0, u1);
+            um = fmaxf(um, fmaxf(u0, u1));
+        }
+        const float q2 = um * um, q4 = q2 * q2;
+        const float gain = fabsf(c.re_a) * (q4 * q2 * um);
+        const float phase = fabsf(c.im_k) * um + fabsf(c.im_p) * (q4 * q4);
+        // (a NaN intensity is not seen by fmaxf: it goes through any form as NaN)
+        if (__all_sync(warp, phase <= 0.03125f && gain < 0.001953125f)) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = screen_k8<0>(v[m], screen_u(v[m], c), c);
+            return;
+        }
+        if (__all_sync(warp, phase <= 0.7853982f && gain < 0.0625f)) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = screen_k8<1>(v[m], screen_u(v[m], c), c);
+            return;
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = apply_screen2(v[m], c, warp);
+}
+
 }  // namespace pr
 
 // ------------------------------------------------------------- row tile --
@@ -286,8 +343,7 @@ __device__ __forceinline__ void row_screens32(C2 (&v)[E], const ScreenCoef<float
                     v[m] = {pr::pk(a.x, b.x), pr::pk(a.y, b.y)};
                 }
             } else {
-#pragma unroll
-                for (int m = 0; m < E; ++m) v[m] = pr::apply_screen2(v[m], sc, warp);
+                pr::apply_screens2(v, sc, warp);
             }
         }
         if (DIAG && rep == 0) {
