@@ -192,6 +192,19 @@ template <typename T> ScreenCoef<T> screen_coef(const nlse_params* p) {
     c.scale = (T)1;
     c.exact = (p->scheme & NLSE_EXACT_SCREEN) ? 1 : 0;
     c.ka = (T)(-2.0 * (p->K - 1) * th[4] * aA);  // (K-1) c_A beta_K dz I_ref^(K-1)
+    // (1 + a)^(-1/(2(K-1))), [(1 + a)^e - 1] / (a e) with e = (K-2)/(K-1) (K = 2:
+    // ln(1 + a)/a) and (K-1) [1 - (1 + a)^(-1/(K-1))] / a by the binomial series
+    const double km1 = p->K > 1 ? p->K - 1.0 : 1.0;
+    auto binom_ratio = [](double x, int j) {  // C(x, j) / x = (x-1)(x-2)..(x-j+1) / j!
+        double r = 1.0;
+        for (int i = 1; i < j; ++i) r *= (x - i) / (i + 1);
+        return r;
+    };
+    for (int j = 1; j <= 4; ++j) {
+        c.ex_amp[j - 1] = (T)(-0.5 / km1 * binom_ratio(-0.5 / km1, j));
+        c.ex_f1[j - 1] = (T)binom_ratio((km1 - 1.0) / km1, j + 1);
+        c.ex_fk[j - 1] = (T)binom_ratio(-1.0 / km1, j + 1);
+    }
     return c;
 }
 

@@ -36,6 +36,9 @@ template <typename T> struct ScreenCoef {
     T ka;          // (K-1) c_A beta_K dz I_ref^(K-1)
     int real_gains;  // 1: re_k = re_p = 0 and im_a = 0 (real gains, e.g. the nominal
                      // ones): the exponent's zero terms are skipped (same values)
+    // power series in a of the exact substep (FP32, |a| <= 2^-7), coefficients of
+    // a^1..a^4 of amp - 1, f1 - 1 and fk - 1 (see apply_screen_exact)
+    T ex_amp[4], ex_f1[4], ex_fk[4];
 };
 
 template <typename T> __device__ __forceinline__ T ipow(T u, int e) {

@@ -280,6 +280,70 @@ template <int FORM> __device__ __forceinline__ C2 screen_k8(C2 v, F2 u, const Sc
 __device__ __forceinline__ F2 screen_u(C2 v, const ScreenCoef<float>& c) {
     return mul(fma(v.re, v.re, mul(v.im, v.im)), bc(c.inv_iref));
 }
+// The exact pointwise substep (kernels.cuh: apply_screen_exact) of all of a
+// thread's values where the warp's largest absorption number |a| is at most 2^-7:
+// amp - 1, f1 and fk by their power series to a^4 (truncation below 1e-10),
+// U = v + v d as in the frozen screen; phases within 1/32 rad (FORM 0) or pi/4.
+// The general form calls log1p, exp, three expm1 and sincos for every value.
+template <int FORM> __device__ __forceinline__ C2 screen_exact2(C2 v, F2 u, const ScreenCoef<float>& c) {
+    F2 uk1, uk;
+    if (c.K == 8) {  // (uniform)
+        const F2 u2 = mul(u, u), u4 = mul(u2, u2);
+        uk1 = mul(mul(u4, u2), u);
+        uk = mul(u4, u4);
+    } else {
+        uk1 = ipow2(u, c.K - 1);
+        uk = mul(uk1, u);
+    }
+    const F2 a = mul(bc(c.ka), uk1), one = bc(1.0f);
+    auto series = [&](const float (&k)[4]) {
+        return mul(a, fma(a, fma(a, fma(a, bc(k[3]), bc(k[2])), bc(k[1])), bc(k[0])));
+    };
+    const F2 em1 = series(c.ex_amp), f1 = add(one, series(c.ex_f1)), fk = add(one, series(c.ex_fk));
+    const F2 im = fma(mul(bc(c.im_k), u), f1, mul(mul(bc(c.im_p), uk), fk));
+    F2 sn, cm1;
+    if constexpr (FORM == 0) sin_cosm1_short2(im, sn, cm1);
+    else sin_cosm1_core2(im, sn, cm1);
+    const F2 dre = fma(em1, cm1, add(em1, cm1)), dim = fma(em1, sn, sn);
+    const F2 ddx = fma(v.re, dre, mul(v.im, neg(dim))), ddy = fma(v.re, dim, mul(v.im, dre));
+    return {add(v.re, ddx), add(v.im, ddy)};
+}
+__device__ __forceinline__ float ipow1(float u, int e) {
+    float r = 1.0f;
+    for (; e > 0; e >>= 1, u *= u)
+        if (e & 1) r *= u;
+    return r;
+}
+template <int E>
+__device__ __forceinline__ void apply_screens_exact2(C2 (&v)[E], const ScreenCoef<float>& c, unsigned warp) {
+    float um = 0.0f;
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        float u0, u1;
+        up(screen_u(v[m], c), u0, u1);
+        um = fmaxf(um, fmaxf(u0, u1));
+    }
+    const float p1 = ipow1(um, c.K - 1);
+    const float phase = fabsf(c.im_k) * um + fabsf(c.im_p) * (p1 * um);  // f1, fk <= 1.01 at |a| <= 2^-7
+    const bool series = fabsf(c.ka) * p1 <= 0.0078125f;
+    if (__all_sync(warp, series && phase <= 0.0309f)) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = screen_exact2<0>(v[m], screen_u(v[m], c), c);
+    } else if (__all_sync(warp, series && phase <= 0.7775f)) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = screen_exact2<1>(v[m], screen_u(v[m], c), c);
+    } else {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            float r0, r1, i0, i1;
+            up(v[m].re, r0, r1);
+            up(v[m].im, i0, i1);
+            const float2 a = apply_screen_exact<float>(make_float2(r0, i0), c.inv_iref, c.im_k, c.im_p, c.ka, c.K);
+            const float2 b = apply_screen_exact<float>(make_float2(r1, i1), c.inv_iref, c.im_k, c.im_p, c.ka, c.K);
+            v[m] = {pk(a.x, b.x), pk(a.y, b.y)};
+        }
+    }
+}
 template <int E> __device__ __forceinline__ void apply_screens2(C2 (&v)[E], const ScreenCoef<float>& c, unsigned warp) {
     if (c.K == 8 && c.real_gains) {  // (uniform)
         float um = 0.0f;
@@ -331,17 +395,7 @@ __device__ __forceinline__ void row_screens32(C2 (&v)[E], const ScreenCoef<float
     for (int rep = 0; rep < sc.reps; ++rep) {
         if (sc.active) {
             if (EXACT && sc.exact) {  // (uniform)
-#pragma unroll
-                for (int m = 0; m < E; ++m) {
-                    float r0, r1, i0, i1;
-                    pr::up(v[m].re, r0, r1);
-                    pr::up(v[m].im, i0, i1);
-                    const float2 a = apply_screen_exact<float>(make_float2(r0, i0), sc.inv_iref, sc.im_k, sc.im_p,
-                                                               sc.ka, sc.K);
-                    const float2 b = apply_screen_exact<float>(make_float2(r1, i1), sc.inv_iref, sc.im_k, sc.im_p,
-                                                               sc.ka, sc.K);
-                    v[m] = {pr::pk(a.x, b.x), pr::pk(a.y, b.y)};
-                }
+                pr::apply_screens_exact2(v, sc, warp);
             } else {
                 pr::apply_screens2(v, sc, warp);
             }
