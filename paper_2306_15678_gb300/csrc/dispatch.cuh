@@ -161,8 +161,9 @@ cudaError_t launch_col_c(const typename vec2<T>::type* src, typename vec2<T>::ty
         constexpr int SMEM = col_smem_bytes<T, N, C>();
         cudaError_t e = ensure_smem<k_col_pass<T, N, C>>(SMEM);
         if (e != cudaSuccess) return e;
-        k_col_pass<T, N, C><<<N / C, threads_per_line<T, N>() * C, SMEM, s>>>(src, dst, tw, px, py, rot);
-        return cudaGetLastError();
+        e = launch_pdl(k_col_pass<T, N, C>, dim3(N / C), dim3(threads_per_line<T, N>() * C), SMEM, s, src, dst, tw, px,
+                       py, rot);
+        return e != cudaSuccess ? e : cudaGetLastError();
     } else {
         return cudaErrorInvalidConfiguration;
     }
@@ -334,22 +335,18 @@ template <typename T, int N> constexpr int col_mask() {
 
 // default column tile: the staged single-column tile where it exists (n >=
 // 512) -- the fastest or within 2 % of the fastest tile at every size
-// measured on GB300 --, else the widest valid tile of at most 512 threads,
-// unless its row segments are shorter than one 32-byte sector, in which case
-// the narrowest valid tile that fills a sector (else the widest valid tile)
+// measured on GB300 --, else the narrowest valid tile whose rows fill a 32-byte
+// sector: the work of a small grid spreads over the most SMs (256^2, where the
+// widest tile of 512 threads ran on 16 SMs: 70 us per column pass)
 template <typename T, int N> constexpr int col_default() {
     constexpr int cs = 2 * (int)sizeof(T);
     if (col_tma_ok<T, N, 1>()) return kColTma | 1;
-    int best = 0;
-    for (int i = 0; i < 5; ++i) {
-        const int c = kColOptions[i];
-        if (((col_mask<T, N>() >> i) & 1) && threads_per_line<T, N>() * c <= 512) best = c;
-    }
-    if (best * cs >= 32) return best;
+    int best = 1;
     for (int i = 0; i < 5; ++i)
-        if (((col_mask<T, N>() >> i) & 1) && kColOptions[i] * cs >= 32) return kColOptions[i];
-    for (int i = 0; i < 5; ++i)
-        if ((col_mask<T, N>() >> i) & 1) best = kColOptions[i];
+        if ((col_mask<T, N>() >> i) & 1) {
+            best = kColOptions[i];
+            if (best * cs >= 32) return best;
+        }
     return best;
 }
 

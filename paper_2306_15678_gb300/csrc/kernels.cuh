@@ -170,6 +170,47 @@ __device__ __forceinline__ double2 apply_screen(double2 v, const ScreenCoef<doub
     return mk<double2>(v.x * pr - v.y * pi, v.x * pi + v.y * pr);
 }
 
+// The screen of all of a thread's values.  FP64, K = 8 and real gains (the
+// nominal case): FP64 instructions bound these passes (GB300 issues them at 1/74
+// of the FP32 rate), and exp and sincos with their general argument reduction
+// were a third of a row pass.  The largest component of the values (found on its
+// high words, by integer operations) bounds |v|^2, so one vote tells when every
+// phase is within 1/32 rad and every gain below 2^-9: Taylor polynomials to below
+// 2^-53 of the factor's change then, applied as v + v d.
+template <int E> __device__ __forceinline__ void apply_screens(double2 (&v)[E], const ScreenCoef<double>& c,
+                                                               unsigned warp) {
+    if (c.K == 8 && c.real_gains) {  // (uniform)
+        int h = 0;
+#pragma unroll
+        for (int m = 0; m < E; ++m)
+            h = max(h, max(__double2hiint(v[m].x) & 0x7fffffff, __double2hiint(v[m].y) & 0x7fffffff));
+        // next high word up: above every component (infinity or NaN stay so)
+        const double top = __hiloint2double(h + 1, 0), u = 2.0 * top * top * c.inv_iref;
+        const double u2 = u * u, u4 = u2 * u2;
+        const double gain = fabs(c.re_a) * (u4 * u2 * u), phase = fabs(c.im_k) * u + fabs(c.im_p) * (u4 * u4);
+        if (__all_sync(warp, phase <= 0.03125 && gain <= 0.001953125)) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                const double w = (v[m].x * v[m].x + v[m].y * v[m].y) * c.inv_iref;
+                const double w2 = w * w, w4 = w2 * w2;
+                const double re = c.re_a * (w4 * w2 * w), im = fma(c.im_p, w4 * w4, c.im_k * w);
+                const double em1 =
+                    fma(re * re, fma(re, fma(re, fma(re, 1.0 / 120, 1.0 / 24), 1.0 / 6), 0.5), re);
+                const double i2 = im * im;
+                const double sn = fma(im * i2, fma(i2, fma(i2, -1.0 / 5040, 1.0 / 120), -1.0 / 6), im);
+                const double cm1 =
+                    i2 * fma(i2, fma(i2, fma(i2, 1.0 / 40320, -1.0 / 720), 1.0 / 24), -0.5);
+                const double dre = fma(em1, cm1, em1 + cm1), dim = fma(em1, sn, sn);
+                v[m] = mk<double2>(fma(v[m].x, dre, fma(-v[m].y, dim, v[m].x)),
+                                   fma(v[m].x, dim, fma(v[m].y, dre, v[m].y)));
+            }
+            return;
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = apply_screen(v[m], c, warp);
+}
+
 // sine and cosine in the precision of the argument
 __device__ __forceinline__ void sincos_(float x, float* s, float* c) { sincosf(x, s, c); }
 __device__ __forceinline__ void sincos_(double x, double* s, double* c) { sincos(x, s, c); }
@@ -366,10 +407,14 @@ template <typename T> struct KCfg {
 
 template <typename T, int N> __host__ __device__ constexpr int elems() { return N < KCfg<T>::E_MAX ? N : KCfg<T>::E_MAX; }
 template <typename T, int N> __host__ __device__ constexpr int threads_per_line() { return N / elems<T, N>(); }
-// rows per block of the row-oriented kernels: at least 128 threads per block
+// rows per block of the row-oriented kernels: a row pair of the state layout (or
+// one row of at least 128 threads), in at least one warp.  Small grids are spread
+// over as many SMs as they have row pairs: at 256^2 in FP64 the slow FP64 units of
+// 64 SMs (4 rows per block) took 40 us per row pass, of 128 SMs half of that.
 template <typename T, int N> __host__ __device__ constexpr int rows_per_block() {
-    return threads_per_line<T, N>() >= 128 ? 1
-           : (128 / threads_per_line<T, N>() > N ? N : 128 / threads_per_line<T, N>());
+    constexpr int tl = threads_per_line<T, N>();
+    constexpr int r = tl >= 128 ? 1 : (tl >= 16 ? 2 : 32 / tl);
+    return r > N ? N : r;
 }
 // minimum resident blocks per SM for a 64-register budget per thread
 template <int THREADS> __host__ __device__ constexpr int min_blocks() {
@@ -463,8 +508,7 @@ __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, type
                         for (int m = 0; m < E; ++m)
                             v[m] = apply_screen_exact<T>(v[m], sc.inv_iref, sc.im_k, sc.im_p, sc.ka, sc.K);
                     } else {
-#pragma unroll
-                        for (int m = 0; m < E; ++m) v[m] = apply_screen(v[m], sc, warp);
+                        apply_screens(v, sc, warp);
                     }
                 }
                 if (DIAG && rep == 0) {
@@ -553,6 +597,8 @@ k_col_pass(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
            typename tab_of<T>::type rot) {
     using V = typename vec2<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
+    pdl_trigger();
+    pdl_wait();
     col_tile<T, N, C, MemPlain>(src, dst, tw, px, py, rot, blockIdx.x * C, reinterpret_cast<V*>(smraw));
 }
 
