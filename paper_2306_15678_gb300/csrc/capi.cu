@@ -1248,7 +1248,8 @@ nlse_status nlse_destroy(nlse_grid* g) {
 // Reverse-mode gradient of J = sum (|U_M|^2 - D)^2 / sum D^2 after M steps
 // (kernels in adjoint.cuh).  The forward run stores the x-spectral state S
 // every `ckpt` steps; the backward sweep recomputes each segment from its
-// checkpoint, keeping the column-pass outputs T_n of the segment, and then
+// checkpoint, keeping the column-pass outputs T_n of the segment (FP32: their
+// inverse row transforms, the fields entering the screens), and then
 // runs the backward row and column passes from the last step of the segment
 // to its first.  All kernels are deterministic, so the recomputed states are
 // bit-identical to the forward ones.
@@ -1439,20 +1440,26 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
         if (cudaMemcpyAsync(state, a->ws + a->lay.ckpt + fb * (size_t)c, fb, cudaMemcpyDeviceToDevice,
                             a->stream) != cudaSuccess)
             return NLSE_ECUDA;
-        for (int s = c0; s < c1; ++s) {  // recompute the segment, keeping T_s
+        for (int s = c0; s < c1; ++s) {  // recompute the segment, keeping T_s or (row_stash) v_s = B_x T_s
             const WT<T>* tws = twiddles_at<T>(a->ws + a->lay.tw, n, s);
+            const bool last = s + 1 == c1;
             if (ks->col_pass(state, seg(s - c0), tws, px_at<T>(a->ws + a->lay.px, n, s),
                              py_at<T>(a->ws + a->lay.py, n, s), rot_for_step<T>(s, nullptr), a->cols,
                              nullptr, 0u, a->stream) != cudaSuccess)
                 return NLSE_ECUDA;
-            if (s + 1 < c1 &&
-                ks->row_pass(seg(s - c0), state, tws, ac.sc, partials, false, a->row_radix, nullptr, 0u, a->stream) !=
+            if (ks->row_stash) {
+                if (ks->row_stash(seg(s - c0), last ? nullptr : state, tws, ac.sc, a->row_radix, a->stream) !=
                     cudaSuccess)
+                    return NLSE_ECUDA;
+            } else if (!last && ks->row_pass(seg(s - c0), state, tws, ac.sc, partials, false, a->row_radix, nullptr,
+                                             0u, a->stream) != cudaSuccess) {
                 return NLSE_ECUDA;
+            }
         }
         for (int s = c1 - 1; s >= c0; --s) {  // reverse the segment with the forward step's constants
             const WT<T>* tws = twiddles_at<T>(a->ws + a->lay.tw, n, s);
-            if (ks->adj_row(gam, seg(s - c0), tws, ac, acc, a->stream) != cudaSuccess) return NLSE_ECUDA;
+            if (ks->adj_row(gam, seg(s - c0), tws, ac, acc, a->row_radix, a->stream) != cudaSuccess)
+                return NLSE_ECUDA;
             if (ks->col_pass(gam, gam, tws, px_at<T>(a->ws + a->lay.pxc, n, s),
                              py_at<T>(a->ws + a->lay.pyc, n, s), conj_of(rot_for_step<T>(s, nullptr)), a->cols,
                              nullptr, 0u, a->stream) != cudaSuccess)

@@ -55,7 +55,12 @@ template <typename T> struct KernelSet {
                            V unrot, cudaStream_t s);
     cudaError_t (*loss_seed)(const V* state, V* gam, const double* target, const W* tw,
                              double seed_scale, double* partials, cudaStream_t s);
-    cudaError_t (*adj_row)(V* gam, const V* tn, const W* tw, AdjCoef<T> ac, double* acc, cudaStream_t s);
+    // backward row pass: tn holds the step's column-pass output T, or (row_stash set)
+    // the field v = B_x T as row_stash left it with row-pass code rad
+    cudaError_t (*adj_row)(V* gam, const V* tn, const W* tw, AdjCoef<T> ac, double* acc, int rad, cudaStream_t s);
+    // row pass of the re-march that also leaves v = B_x seg in seg (dst null: only
+    // that); null where the backward row pass takes T itself
+    cudaError_t (*row_stash)(V* seg, V* dst, const W* tw, ScreenCoef<T> sc, int rad, cudaStream_t s);
     // unnormalised 2D DFT (inverse: conjugate kernel) of a row-major array, in place
     cudaError_t (*dft2)(V* data, const W* tw, bool inverse, cudaStream_t s);
 };
@@ -313,7 +318,7 @@ cudaError_t launch_loss_seed(const typename vec2<T>::type* state, typename vec2<
 
 template <typename T, int N>
 cudaError_t launch_adj_row(typename vec2<T>::type* gam, const typename vec2<T>::type* tn,
-                           const typename tab_of<T>::type* tw, AdjCoef<T> ac, double* acc, cudaStream_t s) {
+                           const typename tab_of<T>::type* tw, AdjCoef<T> ac, double* acc, int, cudaStream_t s) {
     constexpr int RPB = rows_per_block<T, N>(), THREADS = threads_per_line<T, N>() * RPB;
     constexpr int SMEM = row_smem_bytes<T, N>();
     cudaError_t e = ensure_smem<k_adj_row<T, N>>(SMEM);
@@ -366,6 +371,7 @@ template <typename T, int N> KernelSet<T> make_set() {
     k.readout = &launch_readout<T, N>;
     k.loss_seed = &launch_loss_seed<T, N>;
     k.adj_row = &launch_adj_row<T, N>;
+    k.row_stash = nullptr;
     k.dft2 = &launch_dft2<T, N>;
     return k;
 }

@@ -179,25 +179,39 @@ cudaError_t launch_readout32(const float2* state, const float2* tw, float2* fiel
 template <int N>
 cudaError_t launch_loss_seed32(const float2* state, float2* gam, const double* target, const float2* tw,
                                double seed_scale, double* partials, cudaStream_t s) {
-    constexpr int RPB = rows_per_block<float, N>(), THREADS = threads_per_line<float, N>() * RPB;
-    constexpr int SMEM = row_smem_bytes<float, N>();
+    constexpr int THREADS = p_row_threads<N, 16>(), SMEM = p_row_smem<N, 16>(), BLOCKS = N / 2 / p_rows<N, 16>();
     cudaError_t e = ensure_smem<k_loss_seed32<N>>(SMEM);
     if (e != cudaSuccess) return e;
-    k_loss_seed32<N><<<N / RPB, THREADS, SMEM, s>>>(reinterpret_cast<const float4*>(state),
-                                                    reinterpret_cast<float4*>(gam), target, tw, seed_scale, partials);
+    k_loss_seed32<N><<<BLOCKS, THREADS, SMEM, s>>>(reinterpret_cast<const float4*>(state),
+                                                   reinterpret_cast<float4*>(gam), target, twb_of(tw), seed_scale,
+                                                   partials);
     return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t launch_adj_row32(float2* gam, const float2* tn, const float2* tw, AdjCoef<float> ac, double* acc,
-                             cudaStream_t s) {
-    constexpr int RPB = rows_per_block<float, N>(), THREADS = threads_per_line<float, N>() * RPB;
-    constexpr int SMEM = row_smem_bytes<float, N>();
-    cudaError_t e = ensure_smem<k_adj_row32<N>>(SMEM);
+cudaError_t launch_adj_row32(float2* gam, const float2* stash, const float2* tw, AdjCoef<float> ac, double* acc,
+                             int rad, cudaStream_t s) {
+    constexpr int THREADS = p_row_threads<N, 16>(), SMEM = p_row_smem<N, 16>(), BLOCKS = N / 2 / p_rows<N, 16>();
+    cudaError_t e = ensure_smem_carveout<k_adj_row32<N>>(SMEM, carveout_blocks<N>(p_min_blocks<THREADS, 16>()));
     if (e != cudaSuccess) return e;
-    k_adj_row32<N><<<N / RPB, THREADS, SMEM, s>>>(reinterpret_cast<float4*>(gam), reinterpret_cast<const float4*>(tn),
-                                                  tw, ac, acc);
-    return cudaGetLastError();
+    e = launch_pdl(k_adj_row32<N>, dim3(BLOCKS), dim3(THREADS), SMEM, s, reinterpret_cast<float4*>(gam),
+                   reinterpret_cast<const float4*>(stash), twb_of(tw), ac, acc, rad == 8 ? 1 : 0);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int N, int E>
+cudaError_t launch_row_stash32_e(float2* seg, float2* dst, const float2* tw, ScreenCoef<float> sc, cudaStream_t s) {
+    constexpr int THREADS = p_row_threads<N, E>(), SMEM = p_row_smem<N, E>(), BLOCKS = N / 2 / p_rows<N, E>();
+    cudaError_t e = ensure_smem_carveout<k_row_stash32<N, E>>(SMEM, carveout_blocks<N>(p_min_blocks<THREADS, E>()));
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(k_row_stash32<N, E>, dim3(BLOCKS), dim3(THREADS), SMEM, s, reinterpret_cast<float4*>(seg),
+                   reinterpret_cast<float4*>(dst), twb_of(tw), sc);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <int N>
+cudaError_t launch_row_stash32(float2* seg, float2* dst, const float2* tw, ScreenCoef<float> sc, int rad,
+                               cudaStream_t s) {
+    return rad == 8 ? launch_row_stash32_e<N, 8>(seg, dst, tw, sc, s) : launch_row_stash32_e<N, 16>(seg, dst, tw, sc, s);
 }
 
 template <int N, int E> constexpr int col_mask32_e() {
@@ -228,7 +242,7 @@ template <int N> KernelSet<float> make_set32() {
     k.n = N;
     k.row_blocks = N / 2 / p_rows<N, 16>();  // partials of the readout and the radix-16 row pass
     k.row_blocks8 = N / 2 / p_rows<N, 8>();
-    k.adj_blocks = N / rows_per_block<float, N>();
+    k.adj_blocks = k.row_blocks;
     k.col_mask = col_mask32<N>();
     k.col_default = col_default32<N>();
     k.row_radix_mask = 3 | (p_row_staged_ok<N>() ? 4 : 0);
@@ -240,6 +254,7 @@ template <int N> KernelSet<float> make_set32() {
     k.readout = &launch_readout32<N>;
     k.loss_seed = &launch_loss_seed32<N>;
     k.adj_row = &launch_adj_row32<N>;
+    k.row_stash = &launch_row_stash32<N>;
     k.dft2 = &launch_dft2<float, N>;
     return k;
 }

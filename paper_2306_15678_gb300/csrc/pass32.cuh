@@ -251,14 +251,14 @@ __device__ __forceinline__ C2 apply_screen2(C2 v, const ScreenCoef<float>& c, un
     return {add(v.re, ddx), add(v.im, ddy)};
 }
 
-// The screen of all of a thread's values for K = 8 and real gains (the nominal
-// case).  The largest intensity of the warp's values bounds every phase and gain,
-// so one vote picks the polynomials for all of them and the values follow each
-// other without branches (a vote and two branches per value kept the sixteen
-// dependent chains from overlapping).  Short form: phases within 1/32 rad and
+// The screen of all of a thread's values (apply_screens2).  The largest intensity
+// of the warp's values bounds every phase and gain, so one vote picks the
+// polynomials for all of them and the values follow each other without branches
+// (a vote and two branches per value kept the sixteen dependent chains from
+// overlapping).  K = 8 and real gains, the nominal case, have a short form: phases within 1/32 rad and
 // gains below 2^-9 (expm1 to x^3, relative truncation below 4e-10; sin to x^5,
-// cos - 1 to x^6, below 1e-13); middle form: phases within pi/4, gains below
-// 1/16; beyond, value by value (apply_screen2).
+// cos - 1 to x^6, below 1e-13); middle form, for any K and gains: phases within
+// pi/4, gains below 1/16; beyond, value by value (apply_screen2).
 template <int FORM> __device__ __forceinline__ C2 screen_k8(C2 v, F2 u, const ScreenCoef<float>& c) {
     const F2 u2 = mul(u, u), u4 = mul(u2, u2);
     const F2 re = mul(bc(c.re_a), mul(mul(u4, u2), u));
@@ -344,19 +344,41 @@ __device__ __forceinline__ void apply_screens_exact2(C2 (&v)[E], const ScreenCoe
         }
     }
 }
+// exponent of the screen (kernels.cuh: screen_exponent) on both lanes, any K and gains
+__device__ __forceinline__ void screen_exponent2(F2 u, const ScreenCoef<float>& c, F2& re, F2& im) {
+    F2 uk1, uk;
+    if (c.K == 8) {  // (uniform)
+        const F2 u2 = mul(u, u), u4 = mul(u2, u2);
+        uk1 = mul(mul(u4, u2), u);
+        uk = mul(u4, u4);
+    } else {
+        uk1 = ipow2(u, c.K - 1);
+        uk = mul(uk1, u);
+    }
+    re = fma(bc(c.re_k), u, fma(bc(c.re_p), uk, mul(bc(c.re_a), uk1)));
+    im = fma(bc(c.im_k), u, fma(bc(c.im_p), uk, mul(bc(c.im_a), uk1)));
+}
+// (dre, dim) = e^{re + i im} - 1 by the middle form's polynomials
+__device__ __forceinline__ void screen_delta2(F2 re, F2 im, F2& dre, F2& dim) {
+    F2 sn, cm1;
+    const F2 em1 = expm1_core2(re);
+    sin_cosm1_core2(im, sn, cm1);
+    dre = fma(em1, cm1, add(em1, cm1));
+    dim = fma(em1, sn, sn);
+}
 template <int E> __device__ __forceinline__ void apply_screens2(C2 (&v)[E], const ScreenCoef<float>& c, unsigned warp) {
-    if (c.K == 8 && c.real_gains) {  // (uniform)
-        float um = 0.0f;
+    float um = 0.0f;
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-            float u0, u1;
-            up(screen_u(v[m], c), u0, u1);
-            um = fmaxf(um, fmaxf(u0, u1));
-        }
+    for (int m = 0; m < E; ++m) {
+        float u0, u1;
+        up(screen_u(v[m], c), u0, u1);
+        um = fmaxf(um, fmaxf(u0, u1));
+    }
+    // (a NaN intensity is not seen by fmaxf: it goes through any form as NaN)
+    if (c.K == 8 && c.real_gains) {  // (uniform)
         const float q2 = um * um, q4 = q2 * q2;
         const float gain = fabsf(c.re_a) * (q4 * q2 * um);
         const float phase = fabsf(c.im_k) * um + fabsf(c.im_p) * (q4 * q4);
-        // (a NaN intensity is not seen by fmaxf: it goes through any form as NaN)
         if (__all_sync(warp, phase <= 0.03125f && gain < 0.001953125f)) {
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = screen_k8<0>(v[m], screen_u(v[m], c), c);
@@ -365,6 +387,21 @@ template <int E> __device__ __forceinline__ void apply_screens2(C2 (&v)[E], cons
         if (__all_sync(warp, phase <= 0.7853982f && gain < 0.0625f)) {
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = screen_k8<1>(v[m], screen_u(v[m], c), c);
+            return;
+        }
+    } else {
+        const float p1 = ipow1(um, c.K - 1), pk = p1 * um;
+        const float gain = fabsf(c.re_k) * um + fabsf(c.re_p) * pk + fabsf(c.re_a) * p1;
+        const float phase = fabsf(c.im_k) * um + fabsf(c.im_p) * pk + fabsf(c.im_a) * p1;
+        if (__all_sync(warp, phase <= 0.7853982f && gain < 0.0625f)) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                F2 re, im, dre, dim;
+                screen_exponent2(screen_u(v[m], c), c, re, im);
+                screen_delta2(re, im, dre, dim);
+                v[m] = {add(v[m].re, fma(v[m].re, dre, mul(v[m].im, neg(dim)))),
+                        add(v[m].im, fma(v[m].re, dim, mul(v[m].im, dre)))};
+            }
             return;
         }
     }
@@ -877,106 +914,260 @@ k_readout32(const float4* __restrict__ state, const unsigned char* twb, float2* 
 }
 
 // ------------------------------------------------------ adjoint (FP32) --
-// The adjoint's row kernels hold two transforms at once, so they keep the
-// single-line engine of fft.cuh (16 complex per thread, the single-line
-// table at the start of the step's twiddle block) on one row per thread
-// group; a row's element is half of a unit: (re, im) = words (l, 2 + l).
+//
+// The backward sweep re-marches a segment and then needs, at every step, the
+// field v = B_x T entering the step's screen (adjoint.cuh).  The re-march computes
+// it anyway: its row pass (k_row_stash32) writes v over the stored T, in the order
+// its threads hold it (thread t's element m at t + m T_row: contiguous across a
+// warp, no matter which point it is), and the backward row pass (k_adj_row32) reads
+// it back in the same order, so that it runs two transforms instead of three, on
+// the pair engine's mirrored pair of transforms.
 
-__device__ __forceinline__ float2 unit_get(const float4* st, size_t u, int l) {
-    const float* f = reinterpret_cast<const float*>(st + u);
-    return make_float2(f[l], f[2 + l]);
-}
-__device__ __forceinline__ void unit_put(float4* st, size_t u, int l, float2 v) {
-    float* f = reinterpret_cast<float*>(st + u);
-    f[l] = v.x;
-    f[2 + l] = v.y;
-}
-
-// Loss and seed (adjoint.cuh: k_loss_seed) on the unit layout.
-template <int N>
-__global__ void __launch_bounds__(threads_per_line<float, N>() * rows_per_block<float, N>(),
-                                  (min_blocks<threads_per_line<float, N>() * rows_per_block<float, N>()>() + 1) / 2)
-k_loss_seed32(const float4* __restrict__ state, float4* __restrict__ gam, const double* __restrict__ target,
-              const float2* __restrict__ tw, double seed_scale, double* __restrict__ partials) {
-    using V = float2;
-    constexpr int E = elems<float, N>(), TL = threads_per_line<float, N>(), RPB = rows_per_block<float, N>();
-    constexpr int LS = line_stride<float, N, RPB>();
+// Row pass of the re-march: v = B_x seg into seg (stash order), then, unless dst
+// is null (the last step of a segment), the screen and dst = F_x U as
+// k_row_pass32 gives it, bit for bit.
+template <int N, int ER>
+__global__ void __launch_bounds__(p_row_threads<N, ER>(), p_min_blocks<p_row_threads<N, ER>(), ER>())
+k_row_stash32(float4* seg, float4* dst, const unsigned char* twb, ScreenCoef<float> sc) {
+    constexpr int E = p_e<N, ER>(), T = p_tpl<N, ER>(), RP = p_rows<N, ER>();
+    constexpr int LS = pr::pair_line_stride<N, E, RP>();
+    using S = pr::LineSync<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
-    V* smem = reinterpret_cast<V*>(smraw);
-    const int g = row_of_thread<TL, RPB>(), j = lane_in_row<TL, RPB>();
-    const size_t row = (size_t)blockIdx.x * RPB + g;
-    const size_t pu = (row >> 1) * N;
-    const int l = (int)(row & 1);
-    V* sm = smem + g * LS;
-    V v[E];
+    pdl_trigger();
+    pdl_wait();
+    const int g = (int)threadIdx.x / T, t = (int)threadIdx.x % T, j = row_id<N, ER>(t);
+    const size_t row = ((size_t)blockIdx.x * RP + g) * N;
+    C2* sm = reinterpret_cast<C2*>(smraw) + g * LS;
+    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, ER));
+    const unsigned warp = (blockDim.x & 31) == 0 ? 0xffffffffu : __activemask();
+    C2 v[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = unit_get(state, pu + j + m * TL, l);
-    fft_stockham<V, N, E, true>(v, sm, tw, j);
-    const float inv = 1.0f / (float)N;
-    double part = 0.0;
-#pragma unroll
-    for (int m = 0; m < E; ++m) {
-        const V u = cscale(v[m], inv);
-        const double F = (double)(u.x * u.x + u.y * u.y);
-        const double d = F - target[row * N + j + m * TL];
-        part += d * d;
-        const float w = (float)(4.0 * d * seed_scale);  // 4 (F - D) / sum D^2
-        v[m] = cscale(u, w * inv);                       // and the 1/n of G_S = F_x G_U / n
-    }
-    fft_stockham<V, N, E, false>(v, sm, tw, j);
-#pragma unroll
-    for (int m = 0; m < E; ++m) unit_put(gam, pu + j + m * TL, l, v[m]);
-    block_partials<double>(part, 0.0, partials);
-}
-
-// Backward row pass (adjoint.cuh: k_adj_row) on the unit layout.
-template <int N>
-__global__ void __launch_bounds__(threads_per_line<float, N>() * rows_per_block<float, N>(),
-                                  (min_blocks<threads_per_line<float, N>() * rows_per_block<float, N>()>() + 1) / 2)
-k_adj_row32(float4* __restrict__ gam, const float4* __restrict__ tn, const float2* __restrict__ tw,
-            AdjCoef<float> ac, double* __restrict__ acc) {
-    using V = float2;
-    using T = float;
-    constexpr int E = elems<float, N>(), TL = threads_per_line<float, N>(), RPB = rows_per_block<float, N>();
-    constexpr int LS = line_stride<float, N, RPB>();
-    extern __shared__ __align__(16) unsigned char smraw[];
-    V* smem = reinterpret_cast<V*>(smraw);
-    const int g = row_of_thread<TL, RPB>(), j = lane_in_row<TL, RPB>();
-    const size_t row = (size_t)blockIdx.x * RPB + g;
-    const size_t pu = (row >> 1) * N;
-    const int l = (int)(row & 1);
-    V* sm = smem + g * LS;
-    V vt[E], gw[E];
-#pragma unroll
-    for (int m = 0; m < E; ++m) vt[m] = unit_get(tn, pu + j + m * TL, l);
-    fft_stockham<V, N, E, true>(vt, sm, tw, j);  // v = B_x T
-#pragma unroll
-    for (int m = 0; m < E; ++m) gw[m] = unit_get(gam, pu + j + m * TL, l);
-    fft_stockham<V, N, E, true>(gw, sm, tw, j);  // G_U = B_x G_S
-    T th[6] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0};
-    if (ac.sc.active) {
+    for (int m = 0; m < E; ++m) v[m] = pr::swp(UnitPlain::ld(seg + row + j + m * T));
+    auto screen = [&]() {
 #pragma unroll
         for (int m = 0; m < E; ++m) {
-            const V v = vt[m], G = gw[m];
-            const T u = (v.x * v.x + v.y * v.y) * ac.sc.inv_iref;
-            T er, ei, sr, si, uk, uk1;
-            screen_factor_and_slope(u, ac, &er, &ei, &sr, &si, &uk, &uk1);
-            const V w = mk<V>(v.x * er - v.y * ei, v.x * ei + v.y * er);      // U' = v e^s
-            const V c = mk<V>(G.x * w.x + G.y * w.y, G.x * w.y - G.y * w.x);  // conj(G) U'
-            const T q = (T)2 * (c.x * sr - c.y * si);                           // 2 Re(c s')
-            gw[m] = mk<V>(er * G.x + ei * G.y + q * v.x, er * G.y - ei * G.x + q * v.y);
-            th[0] += ac.aK * u * c.y;
-            th[1] += ac.aK * u * c.x;
-            th[2] += ac.aP * uk * c.y;
-            th[3] += ac.aP * uk * c.x;
-            th[4] += ac.aA * uk1 * c.x;
-            th[5] -= ac.aA * uk1 * c.y;
+            v[m] = pr::swp(v[m]);
+            UnitPlain::st(seg + row + t + m * T, v[m]);
+        }
+        if (dst && sc.active) pr::apply_screens2(v, sc, warp);
+    };
+    if constexpr (pr::mirrored(N, E)) {
+        pr::fft_first<N, S>(v, sm, tab, t);
+        screen();
+        if (!dst) return;  // (uniform)
+        pr::fft_second<N, S>(v, sm, tab, t);
+    } else {
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            pr::fft_pair<N, E, S, (ER >= 16)>(v, sm, tab, t);
+            if (half == 0) {
+                screen();
+                if (!dst) return;  // (uniform)
+            }
         }
     }
-    fft_stockham<V, N, E, false>(gw, sm, tw, j);  // G_T = F_x G_v
 #pragma unroll
-    for (int m = 0; m < E; ++m) unit_put(gam, pu + j + m * TL, l, gw[m]);
-    block_accumulate6<T>(th, acc);
+    for (int m = 0; m < E; ++m) UnitPlain::st(dst + row + j + m * T, v[m]);
+}
+
+// Pullback of the screen on one value of both lanes (adjoint.cuh): G = G_U in, G_v
+// out; adds the six theta sums.
+__device__ __forceinline__ C2 adj_value2(C2 v, C2 G, F2 u, F2 re, F2 im, F2 dre, F2 dim, const AdjCoef<float>& a,
+                                         F2 (&th)[6]) {
+    using namespace pr;
+    const ScreenCoef<float>& c = a.sc;
+    F2 k2, k1, k;
+    if (c.K == 8) {  // (uniform)
+        const F2 u2 = mul(u, u), u4 = mul(u2, u2);
+        k2 = mul(u4, u2);
+        k1 = mul(k2, u);
+        k = mul(u4, u4);
+    } else {
+        k2 = c.K >= 2 ? ipow2(u, c.K - 2) : bc(0.0f);
+        k1 = ipow2(u, c.K - 1);
+        k = mul(k1, u);
+    }
+    const float Kf = (float)c.K, K1f = (float)(c.K - 1);
+    const F2 sr = mul(fma(bc(K1f * c.re_a), k2, fma(bc(Kf * c.re_p), k1, bc(c.re_k))), bc(c.inv_iref));
+    const F2 si = mul(fma(bc(K1f * c.im_a), k2, fma(bc(Kf * c.im_p), k1, bc(c.im_k))), bc(c.inv_iref));
+    // U' = v + v d, c = conj(G) U'
+    const F2 wr = add(v.re, fma(v.re, dre, mul(v.im, neg(dim))));
+    const F2 wi = add(v.im, fma(v.re, dim, mul(v.im, dre)));
+    const F2 cr = fma(G.re, wr, mul(G.im, wi)), ci = fma(G.re, wi, mul(neg(G.im), wr));
+    const F2 h = fma(cr, sr, mul(ci, neg(si)));  // Re(c s')
+    const F2 q = add(h, h);
+    const F2 tk = mul(bc(a.aK), u), tp = mul(bc(a.aP), k), ta = mul(bc(a.aA), k1);
+    th[0] = fma(tk, ci, th[0]);
+    th[1] = fma(tk, cr, th[1]);
+    th[2] = fma(tp, ci, th[2]);
+    th[3] = fma(tp, cr, th[3]);
+    th[4] = fma(ta, cr, th[4]);
+    th[5] = fma(ta, neg(ci), th[5]);
+    // conj(e^s) G + q v
+    return {fma(q, v.re, add(G.re, fma(dre, G.re, mul(dim, G.im)))),
+            fma(q, v.im, add(G.im, fma(dre, G.im, mul(neg(dim), G.re))))};
+}
+
+// Six per-thread FP32 sums -> FP64 sums added into acc[block][6], in a fixed order:
+// each warp takes sums 0..5 in turn, its lanes every 32nd thread's value, then a
+// shuffle tree.  (A tree of FP64 shuffles in every warp is 30 FP64 additions per
+// thread: at 8192^2 a fifth of the kernel.)
+template <int THREADS>
+__device__ __forceinline__ void block_accumulate6_f32(const float (&g)[6], double* __restrict__ acc) {
+    __shared__ float red[6][THREADS];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = g[q];
+    __syncthreads();
+    if constexpr (THREADS >= 32) {
+        for (int q = (int)threadIdx.x >> 5; q < 6; q += THREADS / 32) {
+            double s = 0.0;
+            for (int i = (int)threadIdx.x & 31; i < THREADS; i += 32) s += (double)red[q][i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((threadIdx.x & 31) == 0) acc[6 * blockIdx.x + q] += s;
+        }
+    } else {
+        for (int q = threadIdx.x; q < 6; q += THREADS) {
+            double s = 0.0;
+            for (int i = 0; i < THREADS; ++i) s += (double)red[q][i];
+            acc[6 * blockIdx.x + q] += s;
+        }
+    }
+}
+
+// Backward row pass of one step (adjoint.cuh: k_adj_row) on the unit layout:
+// gam <- F_x( adjoint screen( B_x gam ; v ) ), v from the stash; natural != 0: the
+// stash holds v in natural order (written by the radix-8 row pass).
+template <int N>
+__global__ void __launch_bounds__(p_row_threads<N, 16>(), p_min_blocks<p_row_threads<N, 16>(), 16>())
+k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<float> ac, double* __restrict__ acc,
+            int natural) {
+    constexpr int E = p_e<N, 16>(), T = p_tpl<N, 16>(), RP = p_rows<N, 16>();
+    constexpr int LS = pr::pair_line_stride<N, E, RP>();
+    constexpr bool MIR = pr::mirrored(N, E);
+    using S = pr::LineSync<T>;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int g = (int)threadIdx.x / T, t = (int)threadIdx.x % T, j = row_id<N, 16>(t);
+    const size_t row = ((size_t)blockIdx.x * RP + g) * N;
+    C2* sm = reinterpret_cast<C2*>(smraw) + g * LS;
+    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, 16));
+    C2 v[E];
+    pdl_trigger();
+    pdl_wait();
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = pr::swp(UnitPlain::ld(gam + row + j + m * T));
+    F2 th[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) th[q] = pr::bc(0.0f);
+    auto pullback = [&]() {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = pr::swp(v[m]);  // G_U = B_x G_S
+        if (!ac.sc.active) return;  // (uniform)
+        const ScreenCoef<float>& sc = ac.sc;
+        const unsigned warp = (blockDim.x & 31) == 0 ? 0xffffffffu : __activemask();
+        int at = t;
+        if constexpr (MIR)
+            if (natural) at = pr::mid_id<N>(t);
+        const float4* sv = stash + row + at;
+        constexpr int G = E < 4 ? E : 4;  // values whose forms are voted on together
+#pragma unroll
+        for (int m0 = 0; m0 < E; m0 += G) {
+            C2 w[G];
+            float um = 0.0f;
+#pragma unroll
+            for (int i = 0; i < G; ++i) w[i] = UnitPlain::ld(sv + (m0 + i) * T);
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                float u0, u1;
+                pr::up(pr::screen_u(w[i], sc), u0, u1);
+                um = fmaxf(um, fmaxf(u0, u1));
+            }
+            const float p1 = pr::ipow1(um, sc.K - 1), pk = p1 * um;
+            const float gain = fabsf(sc.re_k) * um + fabsf(sc.re_p) * pk + fabsf(sc.re_a) * p1;
+            const float phase = fabsf(sc.im_k) * um + fabsf(sc.im_p) * pk + fabsf(sc.im_a) * p1;
+            const bool poly = __all_sync(warp, phase <= 0.7853982f && gain < 0.0625f);
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                const F2 u = pr::screen_u(w[i], sc);
+                F2 re, im, dre, dim;
+                pr::screen_exponent2(u, sc, re, im);
+                if (poly) {
+                    pr::screen_delta2(re, im, dre, dim);
+                } else {
+                    float r0, r1, i0, i1;
+                    pr::up(re, r0, r1);
+                    pr::up(im, i0, i1);
+                    F2 em1, sn, cm1;
+                    pr::screen_slow2(r0, r1, i0, i1, sc.has_gain, warp, em1, sn, cm1);
+                    dre = pr::fma(em1, cm1, pr::add(em1, cm1));
+                    dim = pr::fma(em1, sn, sn);
+                }
+                v[m0 + i] = adj_value2(w[i], v[m0 + i], u, re, im, dre, dim, ac, th);
+            }
+        }
+    };
+    if constexpr (MIR) {
+        pr::fft_first<N, S>(v, sm, tab, t);
+        pullback();
+        pr::fft_second<N, S>(v, sm, tab, t);
+    } else {
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            pr::fft_pair<N, E, S, true>(v, sm, tab, t);
+            if (half == 0) pullback();
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) UnitPlain::st(gam + row + j + m * T, v[m]);
+    float s6[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) s6[q] = pr::lo(th[q]) + pr::hi(th[q]);
+    block_accumulate6_f32<p_row_threads<N, 16>()>(s6, acc);
+}
+
+// Loss and seed (adjoint.cuh: k_loss_seed) on the unit layout, natural order (the
+// target is row-major): the one-off transforms of the load and the readouts.
+template <int N>
+__global__ void __launch_bounds__(p_row_threads<N, 16>(), p_min_blocks<p_row_threads<N, 16>(), 16>())
+k_loss_seed32(const float4* __restrict__ state, float4* __restrict__ gam, const double* __restrict__ target,
+              const unsigned char* twb, double seed_scale, double* __restrict__ partials) {
+    constexpr int E = p_e<N, 16>(), T = p_tpl<N, 16>(), RP = p_rows<N, 16>();
+    constexpr int LS = pr::pair_line_stride<N, E, RP>();
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int g = (int)threadIdx.x / T, j = (int)threadIdx.x % T;
+    const size_t p = (size_t)blockIdx.x * RP + g;
+    C2* sm = reinterpret_cast<C2*>(smraw) + g * LS;
+    const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_oneoff_off(N));
+    C2 v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = pr::swp(UnitPlain::ld(state + p * N + j + m * T));
+    const float inv = 1.0f / (float)N;
+    const double scale4 = 4.0 * seed_scale;
+    double part = 0.0;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        pr::fft_pair<N, E, pr::LineSync<T>, false>(v, sm, tab, j);
+        if (half == 0) {
+            const F2 iv = pr::bc(inv);
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                const F2 re = pr::mul(v[m].im, iv), im = pr::mul(v[m].re, iv);  // U, swapped back
+                float f[2], w[2];
+                pr::up(pr::fma(re, re, pr::mul(im, im)), f[0], f[1]);
+#pragma unroll
+                for (int l = 0; l < 2; ++l) {
+                    const double d = (double)f[l] - target[(2 * p + l) * N + j + m * T];
+                    part += d * d;
+                    w[l] = (float)(d * scale4) * inv;  // 4 (F - D) / sum D^2, and the 1/n of G_S = F_x G_U / n
+                }
+                const F2 ww = pr::pk(w[0], w[1]);
+                v[m] = {pr::mul(re, ww), pr::mul(im, ww)};
+            }
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) UnitPlain::st(gam + p * N + j + m * T, v[m]);
+    block_partials<double>(part, 0.0, partials);
 }
 
 }  // namespace nlse
