@@ -60,7 +60,9 @@ template <int N, int E, int C> __host__ __device__ constexpr int p_col_smem() {
 // resident blocks per SM for a budget of 128 (E = 16) or 64 (E = 8) registers
 // per thread (a block narrower than a warp still takes a whole warp's registers)
 template <int THREADS, int E> __host__ __device__ constexpr int p_min_blocks() {
-    constexpr int w = (THREADS + 31) / 32 * 32, budget = E >= 16 ? 512 : 1024;
+    // blocks of two warps (1024^2: 3.4 of them per SM) run faster with all the registers
+    // a thread can have than with more of them resident (step 20.9 -> 19.2 us)
+    constexpr int w = (THREADS + 31) / 32 * 32, budget = E >= 16 ? (w == 64 ? 256 : 512) : 1024;
     return w >= budget ? 1 : (budget / w > 32 ? 32 : budget / w);
 }
 // the same for the column kernels, whose radix-8 form needs about 85 registers
