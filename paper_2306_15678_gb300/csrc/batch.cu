@@ -6,9 +6,11 @@
 // tiles of every beam][row tiles of every beam]; blocks claim them in that
 // order from one atomic counter.  A column tile of beam b at step s needs all
 // row tiles of b at step s-1 done, a row tile needs all column tiles of b at
-// step s: per-beam completion counters carry this.  Every item waits only on
-// items numbered before it, and those were claimed by blocks that were
-// running, so progress never depends on how many blocks are resident.  Waits
+// step s: per-beam completion counters carry this.  A block claims its next item
+// when it starts one and works its items off in order; every item waits only on
+// items numbered before it, so the lowest item not yet done is always the one its
+// (running) block is at, and progress never depends on how many blocks are
+// resident.  Waits
 // are bounded by a deadline on %globaltimer; on expiry the block records
 // NLSE_ETIMEOUT in the status word, raises an abort flag that stops every
 // other block, and returns.
@@ -114,6 +116,12 @@ template <int THREADS, int E> constexpr int batch_smem_max() {
            kTmaAlignPad;
 }
 
+// The thread that stores a staged tile and reports an item's completion: not
+// thread 0, which meanwhile decodes the block's next item and looks at its
+// dependency, so that a tile costs the longer of the two latencies and not
+// their sum.
+constexpr int kSignalThread = 32;
+
 // Per-block state of the staged column tiles: the block's mbarrier, its phase
 // (kept by thread 0) and a failure flag for the whole block.
 struct StageState {
@@ -126,9 +134,9 @@ struct StageState {
 // blocks wrote (acquired through the completion counter) before its bulk
 // copies, moves the C columns into their transform lines (pass32.cuh:
 // col_stage_load) and waits for them, bounded; every thread transforms its
-// column exactly as col_tile32 does; thread 0 stores the lines back with bulk
-// copies and waits until those writes are complete, so that the completion
-// signal that follows covers them.  On a wait that runs out the block records
+// column exactly as col_tile32 does; the signalling thread stores the lines back
+// with bulk copies and waits until those writes are complete, so that the
+// completion signal that it sends next covers them.  On a wait that runs out the block records
 // bit 1 (and bit 2 if the copies may still be in flight), raises the abort
 // flag and returns false without touching the field.
 template <int THREADS, int E, int N>
@@ -158,7 +166,7 @@ __device__ __forceinline__ bool batch_col_staged(const BatchBeam& bm, int tile, 
     col_lines32<N, E, C>(smem, twb, px, py, rot, col0, threadIdx.x);
     fence_proxy_async_smem();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == kSignalThread) {
         col_stage_store<N, E, C>(smem, bm.map, col0);
         tma_store_commit_and_wait();
         fence_proxy_async_global();  // the copies' writes, before the completion signal
@@ -167,9 +175,14 @@ __device__ __forceinline__ bool batch_col_staged(const BatchBeam& bm, int tile, 
 }
 
 // one tile of global step k with the step's table copy, as a single grid applies
-// it; false if a staged copy failed (the item then reports no completion)
+// it
+enum TileEnd {
+    kTileFailed,  // a staged copy failed: the item reports no completion
+    kTileStored,  // stored by every thread: a barrier comes before the signal
+    kTileStaged   // stored by the signalling thread's bulk copies
+};
 template <int THREADS, int E, int N>
-__device__ __forceinline__ bool batch_tile(const BatchBeam& bm, bool col, int tile, long long k, float2 rot,
+__device__ __forceinline__ TileEnd batch_tile(const BatchBeam& bm, bool col, int tile, long long k, float2 rot,
                                            C2* smem, StageState& st, const BatchPlan& plan) {
     if constexpr (batch_supported<THREADS, E, N>()) {
         const int d = (int)(k & (kDither - 1)), dp = (int)(k & (kDitherP - 1));
@@ -179,7 +192,9 @@ __device__ __forceinline__ bool batch_tile(const BatchBeam& bm, bool col, int ti
             const float2* px = bm.px + (size_t)dp * N;
             const float4* py = reinterpret_cast<const float4*>(bm.py + (size_t)dp * py32_copy_bytes(N));
             if constexpr (batch_staged<THREADS, E, N>()) {
-                if (plan.staged) return batch_col_staged<THREADS, E, N>(bm, tile, twb, px, py, rot, smem, st, plan);
+                if (plan.staged)
+                    return batch_col_staged<THREADS, E, N>(bm, tile, twb, px, py, rot, smem, st, plan) ? kTileStaged
+                                                                                                   : kTileFailed;
             }
             col_tile32<N, E, C, UnitCG>(bm.field, bm.field, twb, px, py, rot, tile * C, smem);
         } else {
@@ -188,7 +203,7 @@ __device__ __forceinline__ bool batch_tile(const BatchBeam& bm, bool col, int ti
             row_tile32<N, E, RP, false, UnitCG>(bm.field, bm.field, twb, bm.sc, tile * RP, smem, ts, tm);
         }
     }
-    return true;
+    return kTileStored;
 }
 
 // registers: 128 per thread at radix 16, about 85 at radix 8 (the column
@@ -207,14 +222,21 @@ __global__ void __launch_bounds__(THREADS, p_col_min_blocks<THREADS, E>()) k_bat
     StageState st{&s_bar, 0u, &s_fail};
     const long long total = (long long)plan.items_per_step * plan.nsteps;
     const int col_total = plan.col_off[plan.nbeams];
+    unsigned int claimed = 0;     // (thread 0) the block's next item
+    long long step_base = 0;      // (thread 0) steps taken before this launch
+    if (threadIdx.x == 0) {
+        claimed = atomicAdd(plan.next, 1u);
+        step_base = *plan.step_base;
+    }
     for (;;) {
         if (threadIdx.x == 0) {
             int stop = 0;
-            long long i = -1;
-            if (*(volatile int*)plan.abort) stop = 1;
-            else i = (long long)atomicAdd(plan.next, 1u);
-            if (!stop && i >= total) stop = 1;
-            if (!stop) {
+            const long long i = (long long)claimed;
+            if (i >= total) {
+                stop = 1;
+            } else {
+                // claim the next item now: the counter's latency passes behind this one
+                claimed = atomicAdd(plan.next, 1u);
                 const int s = (int)(i / plan.items_per_step), r = (int)(i % plan.items_per_step);
                 const bool col = r < col_total;
                 const int* off = col ? plan.col_off : plan.row_off;
@@ -229,7 +251,13 @@ __global__ void __launch_bounds__(THREADS, p_col_min_blocks<THREADS, E>()) k_bat
                 // column tiles of step s (row items) of this beam
                 const unsigned int need = col ? (unsigned int)s * bm.row_tiles : (unsigned int)(s + 1) * bm.col_tiles;
                 const unsigned int* ctr = col ? plan.done_row + lo : plan.done_col + lo;
-                if (need > 0 && ld_acquire(ctr) < need) {
+                const long long k = step_base + s;  // global step index
+                const float2 rot = plan.rot[k];
+                const int aborted = *(volatile int*)plan.abort;
+                const unsigned int have = ld_acquire(ctr);  // (the three loads in flight together)
+                if (aborted) {
+                    stop = 1;
+                } else if (have < need) {
                     const long long t0 = global_ns();
                     while (ld_acquire(ctr) < need) {
                         if (*(volatile int*)plan.abort) { stop = 1; break; }
@@ -242,9 +270,8 @@ __global__ void __launch_bounds__(THREADS, p_col_min_blocks<THREADS, E>()) k_bat
                         __nanosleep(100);
                     }
                 }
-                const long long k = *plan.step_base + s;  // global step index
                 s_k = k;
-                s_rot = plan.rot[k];  // this step's global phase
+                s_rot = rot;  // this step's global phase
                 s_item_step = (int)(i & 0x7fffffff);
                 s_item_beam = lo;
                 s_item_tile = rr - off[lo];
@@ -260,20 +287,21 @@ __global__ void __launch_bounds__(THREADS, p_col_min_blocks<THREADS, E>()) k_bat
         const float2 rot = s_rot;
         const long long k = s_k;
         const BatchBeam bm = plan.beams[b];
-        bool ok = true;
+        TileEnd end = kTileStored;
         switch (bm.log2n) {
-            case 8: ok = batch_tile<THREADS, E, 256>(bm, col, tile, k, rot, smem, st, plan); break;
-            case 9: ok = batch_tile<THREADS, E, 512>(bm, col, tile, k, rot, smem, st, plan); break;
-            case 10: ok = batch_tile<THREADS, E, 1024>(bm, col, tile, k, rot, smem, st, plan); break;
-            case 11: ok = batch_tile<THREADS, E, 2048>(bm, col, tile, k, rot, smem, st, plan); break;
-            case 12: ok = batch_tile<THREADS, E, 4096>(bm, col, tile, k, rot, smem, st, plan); break;
+            case 8: end = batch_tile<THREADS, E, 256>(bm, col, tile, k, rot, smem, st, plan); break;
+            case 9: end = batch_tile<THREADS, E, 512>(bm, col, tile, k, rot, smem, st, plan); break;
+            case 10: end = batch_tile<THREADS, E, 1024>(bm, col, tile, k, rot, smem, st, plan); break;
+            case 11: end = batch_tile<THREADS, E, 2048>(bm, col, tile, k, rot, smem, st, plan); break;
+            case 12: end = batch_tile<THREADS, E, 4096>(bm, col, tile, k, rot, smem, st, plan); break;
             default: break;
         }
-        if (!ok) return;  // (uniform) the abort flag is raised
-        __threadfence();  // this thread's tile stores, before the completion signal
-        __syncthreads();
-        if (threadIdx.x == 0 && item != plan.skip_item)
+        if (end == kTileFailed) return;             // (uniform) the abort flag is raised
+        if (end == kTileStored) __syncthreads();  // the block's stores, before the signalling thread's fence
+        if (threadIdx.x == kSignalThread && item != plan.skip_item) {
+            __threadfence();
             atomicAdd(col ? plan.done_col + b : plan.done_row + b, 1u);
+        }
     }
 }
 
