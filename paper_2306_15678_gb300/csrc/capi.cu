@@ -677,8 +677,9 @@ cudaError_t finalize(const double* partials, int nparts, double scale, double* o
 namespace {
 
 // scratch of the effective lens: counters, the separable low-pass factors,
-// complex work array (w, its spectrum, w_dif), labels, per-root maximum keys
-// (then the centre list), per-root centres
+// complex work array (w, its spectrum; FP32: then the centre list), labels,
+// per-root maximum keys (FP64: then the centre list), and w_dif (FP32) or per-root
+// centres (FP64: w_dif stays the real part of the work array)
 struct LensScratch {
     size_t ctr, tab, wbuf, lab, key, cen, total;
 };
@@ -687,7 +688,7 @@ LensScratch lens_scratch_layout(int n, int precision) {
     const size_t nn = (size_t)n * n;
     LensScratch L;
     size_t o = 0;
-    L.ctr = o;  o = align256(o + 2 * sizeof(int));
+    L.ctr = o;  o = align256(o + 3 * sizeof(int));
     L.tab = o;  o = align256(o + 2 * (size_t)n * sizeof(double));
     L.wbuf = o; o = align256(o + nn * (precision == NLSE_FP64 ? 16 : 8));
     L.lab = o;  o = align256(o + nn * sizeof(int));
@@ -720,19 +721,20 @@ nlse_status lens_impl(nlse_grid* g, const nlse_lens* ls, unsigned char* sc, int3
     V* wbuf = reinterpret_cast<V*>(sc + SL.wbuf);
     int* lab = reinterpret_cast<int*>(sc + SL.lab);
     unsigned long long* key = reinterpret_cast<unsigned long long*>(sc + SL.key);
-    int* cen = reinterpret_cast<int*>(sc + SL.cen);
-    int* list = reinterpret_cast<int*>(sc + SL.key);  // the keys are done with when the list is gathered
+    constexpr bool F32 = sizeof(T) == 4;
+    int* cen = F32 ? nullptr : reinterpret_cast<int*>(sc + SL.cen);
+    T* wreal = F32 ? reinterpret_cast<T*>(sc + SL.cen) : nullptr;
+    int* list = reinterpret_cast<int*>(F32 ? sc + SL.wbuf : sc + SL.key);
     V* field = at<T>(g, g->lay.aux);
     const auto* tw = twiddles_fixed<T>(g->ws + g->lay.tw);
     cudaStream_t st = g->stream;
-    const int blocks = (int)std::min<size_t>((nn + 255) / 256, 152 * 8);
+    const int blocks = (int)std::min<size_t>((nn / 4 + 255) / 256, 152 * 8);
 
     // the field leaves the state for the scratch half of the grid (row-major,
     // global phase removed) and comes back after the screen
     nlse_status s = readout_any(g, field, nullptr);
     if (s != NLSE_OK) return s;
-    if (cudaMemsetAsync(ctr, 0, 2 * sizeof(int), st) != cudaSuccess) return NLSE_ECUDA;
-    k_lens_fluence<T><<<blocks, 256, 0, st>>>(field, wbuf, nn);
+    if (cudaMemsetAsync(ctr, 0, 3 * sizeof(int), st) != cudaSuccess) return NLSE_ECUDA;
     // separable low-pass factors: fx[p] = exp(-l_dif kx_p^2), fy[q] = exp(-l_dif ky_q^2) / n^2
     std::vector<T> htab(2 * (size_t)n);
     const double kunit = kTwoPi / g->p.L;
@@ -745,29 +747,28 @@ nlse_status lens_impl(nlse_grid* g, const nlse_lens* ls, unsigned char* sc, int3
     T* tab = reinterpret_cast<T*>(sc + SL.tab);
     if (cudaMemcpyAsync(tab, htab.data(), htab.size() * sizeof(T), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return NLSE_ECUDA;
-    cudaError_t e = ks->dft2(wbuf, tw, false, st);
-    if (e != cudaSuccess) return NLSE_ECUDA;
-    k_lens_filter<T><<<blocks, 256, 0, st>>>(wbuf, n, tab, tab + n);
-    e = ks->dft2(wbuf, tw, true, st);
+    cudaError_t e = ks->fluence_lowpass(field, wbuf, wreal, w_dif_out, tab, tab + n, tw, st);
     if (e != cudaSuccess) return NLSE_ECUDA;
 
-    // lenses: regions of Re(wbuf) >= w_l, labelled by their smallest index
-    const int rt = n < 256 ? n : 256;
-    k_hot_runs<T><<<n, rt, 0, st>>>(reinterpret_cast<const T*>(wbuf), n, 2, (T)ls->w_l, lab);
+    // lenses: regions of w_dif >= w_l, labelled by their smallest index; centres: per
+    // lens the smallest index of its largest value
+    const int rt = n / 4 < 256 ? n / 4 : 256;
+    if constexpr (F32) k_hot_runs<T><<<n, rt, 0, st>>>(wreal, n, 1, (T)ls->w_l, lab);
+    else k_hot_runs<T><<<n, rt, 0, st>>>(reinterpret_cast<const T*>(wbuf), n, 2, (T)ls->w_l, lab);
     k_hot_merge<<<blocks, 256, 0, st>>>(lab, n, ls->connectivity, ctr + 1);
-    k_hot_roots<<<blocks, 256, 0, st>>>(lab, n, ctr);
-    k_hot_spread<<<blocks, 256, 0, st>>>(lab, (int)nn);
-    // centres: per lens the smallest index of its largest value
-    if (cudaMemsetAsync(key, 0, nn * sizeof(unsigned long long), st) != cudaSuccess) return NLSE_ECUDA;
-    if (cudaMemsetAsync(cen, 0x7f, nn * sizeof(int), st) != cudaSuccess) return NLSE_ECUDA;
-    k_lens_keymax<T><<<blocks, 256, 0, st>>>(wbuf, lab, key, nn);
-    k_lens_argmax<T><<<blocks, 256, 0, st>>>(wbuf, lab, key, cen, nn);
+    k_hot_roots<true><<<blocks, 256, 0, st>>>(lab, n, ctr, F32 ? list : nullptr, key, cen);
+    if constexpr (F32) {
+        k_hot_spread<<<blocks, 256, 0, st>>>(lab, (int)nn, LensMax32{wreal, key});
+        k_lens_centres<<<32, 256, 0, st>>>(list, ctr, key);
+    } else {
+        k_hot_spread<<<blocks, 256, 0, st>>>(lab, (int)nn, LensMax64{wbuf, key});
+        k_lens_argmax<<<blocks, 256, 0, st>>>(wbuf, lab, key, cen, nn);
+        k_lens_gather<<<blocks, 256, 0, st>>>(lab, cen, list, ctr + 2, nn);  // (the keys are done with)
+    }
     if (cudaGetLastError() != cudaSuccess) return NLSE_ECUDA;
     int hc[2] = {0, 0};
     if (cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NLSE_ECUDA;
-    if (cudaMemsetAsync(ctr, 0, sizeof(int), st) != cudaSuccess) return NLSE_ECUDA;
-    k_lens_gather<<<blocks, 256, 0, st>>>(lab, cen, list, ctr, nn);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return NLSE_ECUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return NLSE_ECUDA;
     if (hc[1] & kHotStatusGaveUp) return NLSE_ETIMEOUT;
     const int nl = hc[0];
     // the list in increasing index order: the order the screen sums the lenses in
@@ -780,7 +781,6 @@ nlse_status lens_impl(nlse_grid* g, const nlse_lens* ls, unsigned char* sc, int3
         if (cudaMemcpyAsync(list, hl.data(), (size_t)nl * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess)
             return NLSE_ECUDA;
     }
-    if (w_dif_out) k_lens_real<T><<<blocks, 256, 0, st>>>(wbuf, w_dif_out, nn);
 
     // Eqs. 5-6 and the screen of Eq. 2
     const double dx = g->p.L / n;
@@ -1060,25 +1060,29 @@ nlse_status nlse_hot_areas(nlse_grid* g, double w_p, int32_t connectivity, int32
     const int nn = n * n;
     const bool f64 = g->p.precision == NLSE_FP64;
     unsigned char* flu = g->ws + g->lay.aux;  // n^2 reals; the labels use the second half of aux
-    int* lab = labels && labels_on_device ? labels : reinterpret_cast<int*>(flu + (size_t)nn * (f64 ? 8 : 4));
+    // the caller's array if the labelling's 16-byte accesses can use it
+    const bool direct = labels && labels_on_device && (reinterpret_cast<uintptr_t>(labels) & 15) == 0;
+    int* lab = direct ? labels : reinterpret_cast<int*>(flu + (size_t)nn * (f64 ? 8 : 4));
     nlse_status st = readout_any(g, nullptr, flu);
     if (st != NLSE_OK) return st;
     // the readout's finalisation has consumed the partials: they hold {count, status} now
     int* word = reinterpret_cast<int*>(dat(g, g->lay.partials));
     if (cudaMemsetAsync(word, 0, 2 * sizeof(int), g->stream) != cudaSuccess) return NLSE_ECUDA;
-    const int rt = n < 256 ? n : 256;
+    const int rt = n / 4 < 256 ? n / 4 : 256;
     if (f64) k_hot_runs<double><<<n, rt, 0, g->stream>>>((const double*)flu, n, 1, w_p, lab);
     else k_hot_runs<float><<<n, rt, 0, g->stream>>>((const float*)flu, n, 1, (float)w_p, lab);
-    const int blocks = std::min((nn + 255) / 256, 152 * 8);
+    const int blocks = std::min((nn / 4 + 255) / 256, 152 * 8);
     k_hot_merge<<<blocks, 256, 0, g->stream>>>(lab, n, connectivity, word + 1);
-    k_hot_roots<<<blocks, 256, 0, g->stream>>>(lab, n, word);
-    k_hot_spread<<<blocks, 256, 0, g->stream>>>(lab, nn);
+    k_hot_roots<false><<<blocks, 256, 0, g->stream>>>(lab, n, word, nullptr, nullptr, nullptr);
+    k_hot_spread<<<blocks, 256, 0, g->stream>>>(lab, nn, HotNothing{});
     if (cudaGetLastError() != cudaSuccess) return NLSE_ECUDA;
     int host_word[2] = {0, 0};
     if (cudaMemcpyAsync(host_word, word, sizeof(host_word), cudaMemcpyDeviceToHost, g->stream) != cudaSuccess)
         return NLSE_ECUDA;
-    if (labels && !labels_on_device &&
-        cudaMemcpyAsync(labels, lab, (size_t)nn * sizeof(int), cudaMemcpyDeviceToHost, g->stream) != cudaSuccess)
+    if (labels && !direct &&
+        cudaMemcpyAsync(labels, lab, (size_t)nn * sizeof(int),
+                        labels_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                        g->stream) != cudaSuccess)
         return NLSE_ECUDA;
     if (cudaStreamSynchronize(g->stream) != cudaSuccess) return NLSE_ECUDA;
     if (host_word[1] & kHotStatusGaveUp) return NLSE_ETIMEOUT;
@@ -1114,16 +1118,16 @@ nlse_status nlse_turbulent_screen(nlse_grid* g, const void* xi, int xi_on_device
     const int blocks = (int)std::min<size_t>((nn + 255) / 256, 152 * 8);
     cudaError_t e;
     if (f64) {
-        k_turb_spectrum<double><<<blocks, 256, 0, g->stream>>>((const double2*)src, (double2*)spec, n, tau, m2max);
-        e = g->k64->dft2((double2*)spec, twiddles_fixed<double>(g->ws + g->lay.tw), true, g->stream);
+        e = g->k64->turb_screen((const double2*)src, (double2*)spec, tau, m2max,
+                                twiddles_fixed<double>(g->ws + g->lay.tw), g->stream);
         if (e == cudaSuccess) {
             k_turb_apply<double><<<blocks, 256, 0, g->stream>>>((double2*)field, (const double2*)spec, c, nn);
             e = g->k64->row_forward((const double2*)field, (double2*)spec, twiddles_fixed<double>(g->ws + g->lay.tw),
                                     g->stream);
         }
     } else {
-        k_turb_spectrum<float><<<blocks, 256, 0, g->stream>>>((const float2*)src, (float2*)spec, n, (float)tau, m2max);
-        e = g->k32->dft2((float2*)spec, twiddles_fixed<float>(g->ws + g->lay.tw), true, g->stream);
+        e = g->k32->turb_screen((const float2*)src, (float2*)spec, (float)tau, m2max,
+                                twiddles_fixed<float>(g->ws + g->lay.tw), g->stream);
         if (e == cudaSuccess) {
             k_turb_apply<float><<<blocks, 256, 0, g->stream>>>((float2*)field, (const float2*)spec, (float)c, nn);
             e = g->k32->row_forward((const float2*)field, (float2*)spec, twiddles_fixed<float>(g->ws + g->lay.tw),
@@ -1181,11 +1185,13 @@ nlse_status nlse_moments(nlse_grid* g, int32_t count, const int32_t* p, const in
         ms.p[k] = k < count ? p[k] : 1;
         ms.q[k] = k < count ? q[k] : 0;
     }
-    const int blocks = (int)std::min<size_t>((nn + 255) / 256, 152 * 4);
+    // blocks of up to 1024 columns, the rows dealt out over about four blocks per SM
+    const int mt = std::min(n / 4, 256), bx = n / 4 / mt, by = std::min(n, 152 * 4 / bx), blocks = bx * by;
     double* part = dat(g, g->lay.diag);
     const double dx = g->p.L / n;
-    if (f64) k_moments<double><<<blocks, 256, 0, g->stream>>>((const double*)flu, n, dx, ms, part);
-    else k_moments<float><<<blocks, 256, 0, g->stream>>>((const float*)flu, n, dx, ms, part);
+    const dim3 grid(bx, by);
+    if (f64) k_moments<double><<<grid, mt, 0, g->stream>>>((const double*)flu, n, dx, ms, part);
+    else k_moments<float><<<grid, mt, 0, g->stream>>>((const float*)flu, n, dx, ms, part);
     if (cudaGetLastError() != cudaSuccess) return NLSE_ECUDA;
     std::vector<double> h((size_t)blocks * kMomMax);
     if (cudaMemcpyAsync(h.data(), part, h.size() * sizeof(double), cudaMemcpyDeviceToHost, g->stream) !=

@@ -61,8 +61,13 @@ template <typename T> struct KernelSet {
     // row pass of the re-march that also leaves v = B_x seg in seg (dst null: only
     // that); null where the backward row pass takes T itself
     cudaError_t (*row_stash)(V* seg, V* dst, const W* tw, ScreenCoef<T> sc, int rad, cudaStream_t s);
-    // unnormalised 2D DFT (inverse: conjugate kernel) of a row-major array, in place
-    cudaError_t (*dft2)(V* data, const W* tw, bool inverse, cudaStream_t s);
+    // turbulent screen: eps = unnormalised inverse 2D DFT of tau xi on the bins within
+    // m2max (row-major; eps may be xi)
+    cudaError_t (*turb_screen)(const V* xi, V* eps, T tau, long long m2max, const W* tw, cudaStream_t s);
+    // low-pass of the fluence of a row-major field: w = F^-1 fx fy F |U|^2, its real
+    // parts to real and real2 (either may be null); w is kept in FP64 only
+    cudaError_t (*fluence_lowpass)(const V* field, V* w, T* real, T* real2, const T* fx, const T* fy, const W* tw,
+                                   cudaStream_t s);
 };
 
 // Raise the dynamic shared-memory limit of one kernel once per device.  The
@@ -269,27 +274,41 @@ cudaError_t launch_row_forward(const typename vec2<T>::type* src, typename vec2<
     return cudaGetLastError();
 }
 
-template <typename T, int N, bool COLS, bool INV>
-cudaError_t launch_dft_lines(typename vec2<T>::type* data, const typename tab_of<T>::type* tw, cudaStream_t s) {
-    constexpr int LPB = dft_lines_per_block<T, N, COLS>(), THREADS = threads_per_line<T, N>() * LPB;
+template <typename T, int N, bool INV, class LD, class ST>
+cudaError_t launch_dft_rows(LD ld, ST st, const typename tab_of<T>::type* tw, cudaStream_t s) {
+    constexpr int LPB = dft_lines_per_block<T, N, false>(), THREADS = threads_per_line<T, N>() * LPB;
     constexpr int SMEM = line_stride<T, N, LPB>() * LPB * (int)sizeof(typename vec2<T>::type);
-    cudaError_t e = ensure_smem<k_dft_lines<T, N, COLS, INV>>(SMEM);
+    cudaError_t e = ensure_smem<k_dft_rows<T, N, INV, LD, ST>>(SMEM);
     if (e != cudaSuccess) return e;
-    k_dft_lines<T, N, COLS, INV><<<N / LPB, THREADS, SMEM, s>>>(data, tw);
+    k_dft_rows<T, N, INV, LD, ST><<<N / LPB, THREADS, SMEM, s>>>(ld, st, tw);
+    return cudaGetLastError();
+}
+template <typename T, int N, bool LOWPASS>
+cudaError_t launch_dft_cols(typename vec2<T>::type* data, const typename tab_of<T>::type* tw, const T* fx, const T* fy,
+                            cudaStream_t s) {
+    constexpr int LPB = dft_lines_per_block<T, N, true>(), THREADS = threads_per_line<T, N>() * LPB;
+    constexpr int SMEM = line_stride<T, N, LPB>() * LPB * (int)sizeof(typename vec2<T>::type);
+    cudaError_t e = ensure_smem<k_dft_cols<T, N, LOWPASS>>(SMEM);
+    if (e != cudaSuccess) return e;
+    k_dft_cols<T, N, LOWPASS><<<N / LPB, THREADS, SMEM, s>>>(data, tw, fx, fy);
     return cudaGetLastError();
 }
 
-template <typename T, int N, bool INV>
-cudaError_t launch_dft2_dir(typename vec2<T>::type* data, const typename tab_of<T>::type* tw, cudaStream_t s) {
-    cudaError_t e = launch_dft_lines<T, N, false, INV>(data, tw, s);
-    if (e != cudaSuccess) return e;
-    return launch_dft_lines<T, N, true, INV>(data, tw, s);
+template <typename T, int N>
+cudaError_t launch_turb_screen(const typename vec2<T>::type* xi, typename vec2<T>::type* eps, T tau, long long m2max,
+                               const typename tab_of<T>::type* tw, cudaStream_t s) {
+    cudaError_t e = launch_dft_rows<T, N, true>(DftLoadSpectrum<T>{xi, tau, m2max}, DftStore<T>{eps}, tw, s);
+    return e != cudaSuccess ? e : launch_dft_cols<T, N, false>(eps, tw, nullptr, nullptr, s);
 }
 
+// FP32 keeps the real parts alone (compact, in `real`), FP64 the complex array
 template <typename T, int N>
-cudaError_t launch_dft2(typename vec2<T>::type* data, const typename tab_of<T>::type* tw, bool inverse,
-                        cudaStream_t s) {
-    return inverse ? launch_dft2_dir<T, N, true>(data, tw, s) : launch_dft2_dir<T, N, false>(data, tw, s);
+cudaError_t launch_fluence_lowpass(const typename vec2<T>::type* field, typename vec2<T>::type* w, T* real, T* real2,
+                                   const T* fx, const T* fy, const typename tab_of<T>::type* tw, cudaStream_t s) {
+    cudaError_t e = launch_dft_rows<T, N, false>(DftLoadFluence<T>{field}, DftStore<T>{w}, tw, s);
+    if (e != cudaSuccess) return e;
+    if ((e = launch_dft_cols<T, N, true>(w, tw, fx, fy, s)) != cudaSuccess) return e;
+    return launch_dft_rows<T, N, true>(DftLoad<T>{w}, DftStoreReal<T, sizeof(T) == 8>{w, real, real2}, tw, s);
 }
 
 template <typename T, int N>
@@ -372,7 +391,8 @@ template <typename T, int N> KernelSet<T> make_set() {
     k.loss_seed = &launch_loss_seed<T, N>;
     k.adj_row = &launch_adj_row<T, N>;
     k.row_stash = nullptr;
-    k.dft2 = &launch_dft2<T, N>;
+    k.turb_screen = &launch_turb_screen<T, N>;
+    k.fluence_lowpass = &launch_fluence_lowpass<T, N>;
     return k;
 }
 

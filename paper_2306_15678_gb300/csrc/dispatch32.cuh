@@ -255,7 +255,8 @@ template <int N> KernelSet<float> make_set32() {
     k.loss_seed = &launch_loss_seed32<N>;
     k.adj_row = &launch_adj_row32<N>;
     k.row_stash = &launch_row_stash32<N>;
-    k.dft2 = &launch_dft2<float, N>;
+    k.turb_screen = &launch_turb_screen<float, N>;
+    k.fluence_lowpass = &launch_fluence_lowpass<float, N>;
     return k;
 }
 

@@ -1,7 +1,7 @@
 // lens.cuh -- kernels of the effective-lens screen (arXiv 2306.15678, Sec. 2,
 // Eqs. 4-6) on a grid's row-major field:
 //   fluence w = |U|^2 into a complex work array, its Gaussian low-pass
-//   w_dif = F^-1 exp(-l_dif k^2) F w (Eq. 4; the transforms are k_dft_lines),
+//   w_dif = F^-1 exp(-l_dif k^2) F w (Eq. 4; turbulence.cuh: k_dft_rows, k_dft_cols),
 //   the lenses = regions of w_dif >= w_l (labelled by the hot-area kernels),
 //   the centre of each lens = its pixel of largest w_dif (first in row-major
 //   order on a tie), and the screen D_f = sum over centres of the radial
@@ -28,60 +28,43 @@ struct LensCoef {
     double r_im[kLensSeg], b[kLensSeg], nu[kLensSeg], eta[kLensSeg];
 };
 
-// wbuf = (|U|^2, 0)
-template <typename T>
-__global__ void k_lens_fluence(const typename vec2<T>::type* __restrict__ field, typename vec2<T>::type* __restrict__ wbuf,
-                               size_t nn) {
-    using V = typename vec2<T>::type;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x) {
-        const V u = field[i];
-        wbuf[i] = mk<V>(u.x * u.x + u.y * u.y, (T)0);
-    }
-}
-
-// spectrum bin (q, p) *= fx[p] fy[q], the separable factors of the low-pass
-// exp(-l_dif (kx^2 + ky^2)) = exp(-l_dif kx^2) exp(-l_dif ky^2), with the 1/n^2
-// of the inverse transform folded into fy (tables built on the host in FP64)
-template <typename T>
-__global__ void k_lens_filter(typename vec2<T>::type* wbuf, int n, const T* __restrict__ fx,
-                              const T* __restrict__ fy) {
-    using V = typename vec2<T>::type;
-    const size_t nn = (size_t)n * n;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x) {
-        const T f = fx[i % n] * fy[i / n];
-        const V v = wbuf[i];
-        wbuf[i] = mk<V>(v.x * f, v.y * f);
-    }
-}
-
 // order-preserving key of a positive value
 __device__ __forceinline__ unsigned long long lens_key(float w) { return (unsigned long long)__float_as_uint(w); }
 __device__ __forceinline__ unsigned long long lens_key(double w) { return (unsigned long long)__double_as_longlong(w); }
 
-// keymax[root] = largest key of the lens (keymax zeroed before)
-template <typename T>
-__global__ void k_lens_keymax(const typename vec2<T>::type* __restrict__ wd, const int* __restrict__ label,
-                              unsigned long long* __restrict__ keymax, size_t nn) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x) {
-        const int root = label[i];
-        if (root >= 0) atomicMax(&keymax[root], lens_key(wd[i].x));
+// What the labels' spreading sweep (hot_areas.cuh) does for each pixel of a lens:
+// key[root] = largest key (reset when the root was found).  FP32 keys carry the
+// pixel below the value, inverted, so that the largest key is the first pixel of
+// the largest value; FP64 keys fill the word, and k_lens_argmax finds the pixel.
+struct LensMax32 {
+    const float* w;
+    unsigned long long* key;
+    __device__ __forceinline__ void operator()(int root, int i) const {
+        atomicMax(&key[root], (lens_key(w[i]) << 32) | (0xffffffffu - (unsigned)i));
     }
-}
-
-// centre[root] = smallest index holding the lens's largest value (centre set
-// to INT_MAX-like values before)
-template <typename T>
-__global__ void k_lens_argmax(const typename vec2<T>::type* __restrict__ wd, const int* __restrict__ label,
-                              const unsigned long long* __restrict__ keymax, int* __restrict__ centre, size_t nn) {
+};
+struct LensMax64 {
+    const double2* w;
+    unsigned long long* key;
+    __device__ __forceinline__ void operator()(int root, int i) const { atomicMax(&key[root], lens_key(w[i].x)); }
+};
+// centre[root] = smallest index holding the lens's largest value
+static __global__ void k_lens_argmax(const double2* __restrict__ wd, const int* __restrict__ label,
+                                     const unsigned long long* __restrict__ keymax, int* __restrict__ centre, size_t nn) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x) {
         const int root = label[i];
         if (root >= 0 && lens_key(wd[i].x) == keymax[root]) atomicMin(&centre[root], (int)i);
     }
 }
-
-// list of the centres, in no particular order (the host sorts it)
-__global__ void k_lens_gather(const int* __restrict__ label, const int* __restrict__ centre, int* __restrict__ list,
-                              int* __restrict__ count, size_t nn) {
+// FP32: list of roots -> list of centres, in no particular order (the host sorts it)
+static __global__ void k_lens_centres(int* list, const int* __restrict__ count,
+                                      const unsigned long long* __restrict__ key) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < *count; k += gridDim.x * blockDim.x)
+        list[k] = (int)(0xffffffffu - (unsigned)key[list[k]]);
+}
+// FP64: the same from the labels and the per-root centres
+static __global__ void k_lens_gather(const int* __restrict__ label, const int* __restrict__ centre,
+                                     int* __restrict__ list, int* __restrict__ count, size_t nn) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x)
         if (label[i] == (int)i) list[atomicAdd(count, 1)] = centre[i];
 }
@@ -158,13 +141,6 @@ __global__ void __launch_bounds__(256) k_lens_apply(typename vec2<T>::type* fiel
     const size_t i = (size_t)y * n + x;
     const V u = field[i];
     field[i] = mk<V>((T)(amp * ((double)u.x * cs - (double)u.y * sn)), (T)(amp * ((double)u.x * sn + (double)u.y * cs)));
-}
-
-// out = Re(wbuf): w_dif for callers that want it
-template <typename T>
-__global__ void k_lens_real(const typename vec2<T>::type* __restrict__ wbuf, T* __restrict__ out, size_t nn) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x)
-        out[i] = wbuf[i].x;
 }
 
 }  // namespace nlse
