@@ -593,9 +593,8 @@ template <typename T> nlse_status readout_impl(nlse_grid* g, VT<T>* field_out, T
                                 partials, unrot_value<T>(g->theta), g->stream);
     if (e != cudaSuccess) return NLSE_ECUDA;
     const double dx = g->p.L / g->p.n;
-    k_finalize<<<1, 256, 0, g->stream>>>(partials, ks->row_blocks, dx * dx, dat(g, g->lay.readout),
-                                         reinterpret_cast<int*>(g->ws + g->lay.status));
-    return cuerr(cudaGetLastError());
+    return cuerr(launch_finalize(partials, ks->row_blocks, dx * dx, dat(g, g->lay.readout),
+                                 reinterpret_cast<int*>(g->ws + g->lay.status), g->stream));
 }
 
 nlse_status readout_any(nlse_grid* g, void* field_out, void* flu_out) {
@@ -665,8 +664,7 @@ float2 rot_step_f32(long long k, double* applied) { return ::rot_for_step<float>
 
 cudaError_t finalize(const double* partials, int nparts, double scale, double* out, int* status,
                      cudaStream_t s) {
-    k_finalize<<<1, 256, 0, s>>>(partials, nparts, scale, out, status);
-    return cudaGetLastError();
+    return launch_finalize(partials, nparts, scale, out, status, s);
 }
 
 }  // namespace detail

@@ -145,6 +145,13 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, int smem, cu
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// k_finalize on one block of 256
+inline cudaError_t launch_finalize(const double* partials, int nparts, double scale, double* out, int* status,
+                                   cudaStream_t s) {
+    const cudaError_t e = launch_pdl(k_finalize, dim3(1), dim3(256), 0, s, partials, nparts, scale, out, status);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <typename T, int N>
 cudaError_t launch_row_pass(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
                             const typename tab_of<T>::type* tw, ScreenCoef<T> sc, double* partials,
@@ -270,8 +277,8 @@ cudaError_t launch_row_forward(const typename vec2<T>::type* src, typename vec2<
     constexpr int SMEM = row_smem_bytes<T, N>();
     cudaError_t e = ensure_smem<k_row_forward<T, N>>(SMEM);
     if (e != cudaSuccess) return e;
-    k_row_forward<T, N><<<N / RPB, THREADS, SMEM, s>>>(src, dst, tw);
-    return cudaGetLastError();
+    e = launch_pdl(k_row_forward<T, N>, dim3(N / RPB), dim3(THREADS), SMEM, s, src, dst, tw);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T, int N, bool INV, class LD, class ST>
@@ -319,8 +326,9 @@ cudaError_t launch_readout(const typename vec2<T>::type* state, const typename t
     constexpr int SMEM = row_smem_bytes<T, N>();
     cudaError_t e = ensure_smem<k_readout<T, N>>(SMEM);
     if (e != cudaSuccess) return e;
-    k_readout<T, N><<<N / RPB, THREADS, SMEM, s>>>(state, tw, field_out, flu_out, partials, unrot);
-    return cudaGetLastError();
+    e = launch_pdl(k_readout<T, N>, dim3(N / RPB), dim3(THREADS), SMEM, s, state, tw, field_out, flu_out, partials,
+                   unrot);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T, int N>

@@ -161,8 +161,9 @@ template <int N> cudaError_t launch_row_forward32(const float2* src, float2* dst
     constexpr int THREADS = p_row_threads<N, 16>(), SMEM = p_row_smem<N, 16>(), BLOCKS = N / 2 / p_rows<N, 16>();
     cudaError_t e = ensure_smem<k_row_forward32<N>>(SMEM);
     if (e != cudaSuccess) return e;
-    k_row_forward32<N><<<BLOCKS, THREADS, SMEM, s>>>(src, reinterpret_cast<float4*>(dst), twb_of(tw));
-    return cudaGetLastError();
+    e = launch_pdl(k_row_forward32<N>, dim3(BLOCKS), dim3(THREADS), SMEM, s, src, reinterpret_cast<float4*>(dst),
+                   twb_of(tw));
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int N>
@@ -171,9 +172,9 @@ cudaError_t launch_readout32(const float2* state, const float2* tw, float2* fiel
     constexpr int THREADS = p_row_threads<N, 16>(), SMEM = p_row_smem<N, 16>(), BLOCKS = N / 2 / p_rows<N, 16>();
     cudaError_t e = ensure_smem<k_readout32<N>>(SMEM);
     if (e != cudaSuccess) return e;
-    k_readout32<N><<<BLOCKS, THREADS, SMEM, s>>>(reinterpret_cast<const float4*>(state), twb_of(tw), field_out,
-                                                 flu_out, partials, unrot);
-    return cudaGetLastError();
+    e = launch_pdl(k_readout32<N>, dim3(BLOCKS), dim3(THREADS), SMEM, s, reinterpret_cast<const float4*>(state),
+                   twb_of(tw), field_out, flu_out, partials, unrot);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int N>

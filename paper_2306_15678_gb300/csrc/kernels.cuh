@@ -248,6 +248,18 @@ __device__ __noinline__ typename vec2<T>::type apply_screen_exact(typename vec2<
     return mk<typename vec2<T>::type>(v.x * pr - v.y * pi, v.x * pi + v.y * pr);
 }
 
+// Programmatic dependent launch between the passes of the march, and of the load
+// prologue, the readouts and their finalisation: a pass lets the next one's blocks
+// be scheduled when its own are about to store, and waits for the full completion,
+// with its memory, of the pass before it ahead of any access to the field.  Both are
+// no-ops for a kernel launched without the attribute.  (Triggered at their start, the
+// blocks of several passes to come pile up on the SMs that are free at the time,
+// and the blocks of a pass are then spread unevenly over the SMs: 1024^2 19.2 against
+// 14.8 us per step, 512^2 12.1 against 10.7; 256^2 in FP64, bound by each SM's slow
+// FP64 units, up to 100 against 40.)
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------- reductions --
 
 // Per-thread (sum, max) -> per-block FP64 partials, fixed combination order.
@@ -374,6 +386,7 @@ static __global__ void __launch_bounds__(256) k_finalize(const double* __restric
                                                   double scale, double* __restrict__ out,
                                                   int* __restrict__ status) {
     __shared__ double scratch[512];
+    pdl_wait();
     block_finalize(partials, nparts, scale, out, status, scratch);
 }
 
@@ -522,6 +535,7 @@ __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, type
             }
         }
     }
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + sidx<N>(row, j + m * TL), v[m]);
 }
@@ -558,17 +572,10 @@ __device__ __forceinline__ void col_tile(const typename vec2<T>::type* src, type
         }
     }
     conj_all(v);
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + sidx<N>(j + m * TL, col), v[m]);
 }
-
-// Programmatic dependent launch between the passes of the march: a pass lets
-// the next pass's blocks be scheduled as soon as all of its own blocks are
-// running (their set-up then overlaps its last wave), and waits for the full
-// completion, with its memory, of the pass before it ahead of any access to the
-// field.  Both are no-ops for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Row pass kernel of the march; with DIAG the block also reduces sum |U|^2 and
 // max |U|^2 of its rows into partials.
@@ -581,7 +588,6 @@ k_row_pass(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
     constexpr int RPB = rows_per_block<T, N>();
     extern __shared__ __align__(16) unsigned char smraw[];
     T tsum = (T)0, tmax = (T)0;
-    pdl_trigger();
     pdl_wait();
     row_tile<T, N, RPB, DIAG, MemPlain>(src, dst, tw, sc, blockIdx.x * RPB, reinterpret_cast<V*>(smraw),
                                         tsum, tmax);
@@ -597,7 +603,6 @@ k_col_pass(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
            typename tab_of<T>::type rot) {
     using V = typename vec2<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
-    pdl_trigger();
     pdl_wait();
     col_tile<T, N, C, MemPlain>(src, dst, tw, px, py, rot, blockIdx.x * C, reinterpret_cast<V*>(smraw));
 }
@@ -617,9 +622,11 @@ k_row_forward(const typename vec2<T>::type* __restrict__ src, typename vec2<T>::
     const int g = row_of_thread<TL, RPB>(), j = lane_in_row<TL, RPB>();
     const size_t row = (size_t)blockIdx.x * RPB + g;
     V v[E];
+    pdl_wait();
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = src[row * N + j + m * TL];
     fft_stockham<V, N, E, false>(v, smem + g * LS, tw, j);
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) dst[sidx<N>(row, j + m * TL)] = v[m];
 }
@@ -641,9 +648,11 @@ k_readout(const typename vec2<T>::type* __restrict__ state, const typename tab_o
     const int g = row_of_thread<TL, RPB>(), j = lane_in_row<TL, RPB>();
     const size_t row = (size_t)blockIdx.x * RPB + g;
     V v[E];
+    pdl_wait();
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = state[sidx<N>(row, j + m * TL)];
     fft_stockham<V, N, E, true>(v, smem + g * LS, tw, j);
+    pdl_trigger();
     const T inv = (T)1 / (T)N;
     T tsum = (T)0, tmax = (T)0;
 #pragma unroll

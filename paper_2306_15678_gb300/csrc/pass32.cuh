@@ -136,6 +136,7 @@ struct UnitPlain {
         pr::up(v.im, f.z, f.w);
         *p = f;
     }
+    __device__ __forceinline__ static void stores_next() { pdl_trigger(); }
 };
 struct UnitCG {
     static constexpr bool kExactScreen = false;
@@ -149,6 +150,7 @@ struct UnitCG {
         pr::up(v.im, f.z, f.w);
         __stcg(p, f);
     }
+    __device__ __forceinline__ static void stores_next() {}
 };
 
 // --------------------------------------------------------------- screen --
@@ -499,6 +501,7 @@ __device__ __forceinline__ void row_tile32(const float4* src, float4* dst, const
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = pr::swp(M::ld(src + row + j + m * T));  // B_x = swap F_x swap
     row_body32<N, ER, DIAG, M::kExactScreen>(v, sm, tab, sc, t, tsum, tmax);
+    M::stores_next();
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + row + j + m * T, v[m]);
 }
@@ -592,7 +595,6 @@ k_row_pass32(const float4* src, float4* dst, const unsigned char* twb, ScreenCoe
              double* __restrict__ partials) {
     extern __shared__ __align__(16) unsigned char smraw[];
     float tsum = 0.0f, tmax = 0.0f;
-    pdl_trigger();
     pdl_wait();
     row_tile32<N, ER, p_rows<N, ER>(), DIAG, UnitPlain>(src, dst, twb, sc, blockIdx.x * p_rows<N, ER>(),
                                                          reinterpret_cast<C2*>(smraw), tsum, tmax);
@@ -668,7 +670,6 @@ k_row_pass32_pf(const float4* src, float4* dst, const unsigned char* twb, Screen
 #pragma unroll 1
         for (int r = 0; r < 16; ++r) bulk_load_1d(line + r * RS, src + (size_t)p * N + r * T, T * 16, &bar);
     };
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) {
         s_fail = 0;
@@ -700,6 +701,7 @@ k_row_pass32_pf(const float4* src, float4* dst, const unsigned char* twb, Screen
             }
         };
         row_body32<N, 16, DIAG, true, LineFree<decltype(fetch_next)>>(v, line, tab, sc, t, tsum, tmax, {fetch_next});
+        if (next >= NP) pdl_trigger();
 #pragma unroll
         for (int m = 0; m < E; ++m) UnitPlain::st(dst + (size_t)p * N + j + m * T, v[m]);
         if constexpr (DIAG) block_partials32_at(tsum, tmax, partials, p);
@@ -720,6 +722,7 @@ __device__ __forceinline__ void col_tile32(const float4* src, float4* dst, const
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = M::ld(src + (size_t)(j + m * T) * N + col);
     col_body32<N, EC, pr::LineSync<T, C>>(v, smem + c * LS, twb, px, py, rot, col, j);
+    M::stores_next();
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + (size_t)(j + m * T) * N + col, v[m]);
 }
@@ -730,7 +733,6 @@ __global__ void __launch_bounds__(p_col_tpl<N, EC>() * C, p_col_min_blocks<p_col
 k_col_pass32(const float4* src, float4* dst, const unsigned char* twb, const float2* __restrict__ px,
              const float4* __restrict__ py, float2 rot) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    pdl_trigger();
     pdl_wait();
     col_tile32<N, EC, C, UnitPlain>(src, dst, twb, px, py, rot, blockIdx.x * C, reinterpret_cast<C2*>(smraw));
 }
@@ -829,7 +831,6 @@ k_col_pass32_tma(const __grid_constant__ CUtensorMap mload, const __grid_constan
     const uint32_t pad = (kTmaAlign - (smem_u32(smraw) & (kTmaAlign - 1))) & (kTmaAlign - 1);
     C2* smem = reinterpret_cast<C2*>(smraw + pad);
     const int col0 = blockIdx.x * C;
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) {
         s_fail = 0;
@@ -846,6 +847,7 @@ k_col_pass32_tma(const __grid_constant__ CUtensorMap mload, const __grid_constan
     __syncthreads();
     if (s_fail) return;  // (uniform)
     col_lines32<N, EC, C>(smem, twb, px, py, rot, col0, threadIdx.x);
+    pdl_trigger();
     fence_proxy_async_smem();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -866,12 +868,14 @@ k_row_forward32(const float2* __restrict__ src, float4* __restrict__ dst, const 
     const size_t p = (size_t)blockIdx.x * RP + g;
     const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_oneoff_off(N));
     C2 v[E];
+    pdl_wait();
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const float2 a = src[(2 * p) * N + j + m * T], b = src[(2 * p + 1) * N + j + m * T];
         v[m] = {pr::pk(a.x, b.x), pr::pk(a.y, b.y)};
     }
     pr::fft_pair<N, E, pr::LineSync<T>, false>(v, reinterpret_cast<C2*>(smraw) + g * LS, tab, j);
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) UnitPlain::st(dst + p * N + j + m * T, v[m]);
 }
@@ -890,9 +894,11 @@ k_readout32(const float4* __restrict__ state, const unsigned char* twb, float2* 
     const size_t p = (size_t)blockIdx.x * RP + g;
     const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_oneoff_off(N));
     C2 v[E];
+    pdl_wait();
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = pr::swp(UnitPlain::ld(state + p * N + j + m * T));
     pr::fft_pair<N, E, pr::LineSync<T>, false>(v, reinterpret_cast<C2*>(smraw) + g * LS, tab, j);
+    pdl_trigger();
     const float inv = 1.0f / (float)N;
     float tsum = 0.0f, tmax = 0.0f;
 #pragma unroll
@@ -935,7 +941,6 @@ k_row_stash32(float4* seg, float4* dst, const unsigned char* twb, ScreenCoef<flo
     constexpr int LS = pr::pair_line_stride<N, E, RP>();
     using S = pr::LineSync<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
-    pdl_trigger();
     pdl_wait();
     const int g = (int)threadIdx.x / T, t = (int)threadIdx.x % T, j = row_id<N, ER>(t);
     const size_t row = ((size_t)blockIdx.x * RP + g) * N;
@@ -968,6 +973,7 @@ k_row_stash32(float4* seg, float4* dst, const unsigned char* twb, ScreenCoef<flo
             }
         }
     }
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) UnitPlain::st(dst + row + j + m * T, v[m]);
 }
@@ -1054,7 +1060,6 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
     C2* sm = reinterpret_cast<C2*>(smraw) + g * LS;
     const RowTab* tab = reinterpret_cast<const RowTab*>(twb + tw32_row_off(N, 16));
     C2 v[E];
-    pdl_trigger();
     pdl_wait();
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = pr::swp(UnitPlain::ld(gam + row + j + m * T));
@@ -1119,6 +1124,7 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
             if (half == 0) pullback();
         }
     }
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) UnitPlain::st(gam + row + j + m * T, v[m]);
     float s6[6];

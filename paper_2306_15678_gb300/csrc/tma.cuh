@@ -145,7 +145,6 @@ k_col_pass_tma(const __grid_constant__ CUtensorMap mload, const __grid_constant_
     const int col0 = blockIdx.x * C;
     // stage index of (y, c): [y/2][c][y mod 2]
     auto st = [](int y, int c) { return C == 1 ? y : ((y >> 1) * C + c) * 2 + (y & 1); };
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) {
         s_fail = 0;
@@ -181,6 +180,7 @@ k_col_pass_tma(const __grid_constant__ CUtensorMap mload, const __grid_constant_
         }
     }
     conj_all(v);
+    pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) stage[st(j + m * TL, c)] = v[m];
     fence_proxy_async_smem();
