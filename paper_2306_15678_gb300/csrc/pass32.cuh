@@ -60,15 +60,19 @@ template <int N, int E, int C> __host__ __device__ constexpr int p_col_smem() {
 // resident blocks per SM for a budget of 128 (E = 16) or 64 (E = 8) registers
 // per thread (a block narrower than a warp still takes a whole warp's registers)
 template <int THREADS, int E> __host__ __device__ constexpr int p_min_blocks() {
-    // blocks of two warps (1024^2: 3.4 of them per SM) run faster with all the registers
-    // a thread can have than with more of them resident (step 20.9 -> 19.2 us)
-    constexpr int w = (THREADS + 31) / 32 * 32, budget = E >= 16 ? (w == 64 ? 256 : 512) : 1024;
+    // blocks of two warps (1024^2: 3.4 of them per SM), and the radix-8 rows of the small
+    // grids, run faster with all the registers a thread can have than with more of
+    // them resident (1024^2 step 20.9 -> 19.2 us)
+    constexpr int w = (THREADS + 31) / 32 * 32, budget = w == 64 || (E < 16 && w == 32) ? 256 : E >= 16 ? 512 : 1024;
     return w >= budget ? 1 : (budget / w > 32 ? 32 : budget / w);
 }
 // the same for the column kernels, whose radix-8 form needs about 85 registers
 // per thread (the propagator and cross-lane factors on top of the transform)
 template <int THREADS, int E> __host__ __device__ constexpr int p_col_min_blocks() {
-    constexpr int w = (THREADS + 31) / 32 * 32, budget = E >= 16 ? 512 : 768;
+    // blocks of one or two warps serve the small grids, which leave an SM a few of them:
+    // no register limit (at 128 the transforms shorter than 512 points spilled; 256^2
+    // step 8.8 -> 7.1 us, 512^2 10.3 -> 9.4, 1024^2 14.8 -> 14.6)
+    constexpr int w = (THREADS + 31) / 32 * 32, budget = w <= 64 ? 256 : E >= 16 ? 512 : 768;
     return w >= budget ? 1 : (budget / w > 32 ? 32 : budget / w);
 }
 
