@@ -1209,7 +1209,7 @@ nlse_status nlse_history(nlse_grid* g, double* power, double* peak, int32_t capa
     if (flush_diag_any(g) != NLSE_OK) return NLSE_ECUDA;
     const int64_t have = g->hist_count < kHistCap ? g->hist_count : kHistCap;
     const int64_t first = g->hist_count - have;
-    std::vector<double> buf(2 * (size_t)kHistCap);
+    std::vector<double> buf(2 * (size_t)have);  // the whole ring once it has wrapped, else its start
     if (have > 0) {
         if (cudaMemcpyAsync(buf.data(), g->ws + g->lay.hist, buf.size() * sizeof(double),
                             cudaMemcpyDeviceToHost, g->stream) != cudaSuccess)
