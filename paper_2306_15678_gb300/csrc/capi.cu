@@ -41,7 +41,7 @@ size_t py_bytes(int n, int precision) {
     return precision == NLSE_FP64 ? (size_t)n * 16 : (size_t)kDitherP * py32_copy_bytes(n);
 }
 // bytes of the twiddle region: FP64 one pass-major table of n 16-byte
-// entries; FP32 kDither twiddle blocks and the one-off table (pass32.cuh)
+// entries; FP32 kDither twiddle blocks and the one-off tables (pass32.cuh)
 size_t tw_region_bytes(int n, int precision) {
     return precision == NLSE_FP64 ? (size_t)n * 16 : tw32_region_bytes(n);
 }
@@ -265,6 +265,11 @@ template <typename T> const typename tab_of<T>::type* twiddles_at(const unsigned
 template <typename T> const typename tab_of<T>::type* twiddles_fixed(const unsigned char* table) {
     return reinterpret_cast<const typename tab_of<T>::type*>(table);
 }
+// the single-line table of fft.cuh for transforms of row-major arrays
+template <typename T> const typename tab_of<T>::type* twiddles_line(const unsigned char* table, int n) {
+    if (sizeof(T) == 4) table += tw32_line_off(n);
+    return reinterpret_cast<const typename tab_of<T>::type*>(table);
+}
 // copies of the propagator tables for step k
 template <typename T> const typename tab_of<T>::type* px_at(const unsigned char* table, int n, int64_t k) {
     if (sizeof(T) == 4) table += (size_t)(k & (kDitherP - 1)) * n * 8;
@@ -332,8 +337,8 @@ void fused_table(int l, std::vector<double>& out) {
     }
 }
 
-// FP32 tables of one grid: kDither twiddle blocks (single-line table, row and
-// column pair tables), P_x (kDitherP x n entries) and P_y with the cross-lane
+// FP32 tables of one grid: kDither twiddle blocks (row and column pair tables)
+// with the one-off tables, P_x (kDitherP x n entries) and P_y with the cross-lane
 // factors W_n^k (kDitherP x (n/2 pair entries (k, k + n/2), n/2 entries));
 // every component of every entry dithered independently.  The cross-lane and propagator factors e^{i phi} are
 // stored as (cos phi - 1, sin phi) (pass32.cuh), cos phi - 1 = -2 sin^2(phi/2)
@@ -384,12 +389,10 @@ void build_tables_f32(const nlse_params* p, HostTables32& t) {
             dither_into(dp[2 * (k + h) + c], kTabPy, k + h, c, t.py.data() + 4 * q + 2 * c + 1, pyf);
             dither_into(cross[2 * k + c], kTabCross, k, c, t.py.data() + 4 * h + 2 * q + c, pyf);
         }
-    // twiddle blocks: kDither copies (stride cb bytes), then the one-off table
+    // twiddle blocks: kDither copies (stride cb bytes), then the one-off tables
     const size_t cb = tw32_copy_bytes(n), cbf = cb / 4;
     t.tw.assign(tw32_region_bytes(n), 0);
     float* tw = reinterpret_cast<float*>(t.tw.data());
-    for (size_t e = 0; e < single.size() / 2; ++e)
-        for (int c = 0; c < 2; ++c) dither_into(single[2 * e + c], kTabTwiddle, e, c, tw + 2 * e + c, cbf);
     const uint64_t pid[4] = {kTabRowFused, kTabColFused, kTabRowPair8, kTabColPair8};
     const size_t poff[4] = {tw32_row_off(n, 16), tw32_col_off(n, 16), tw32_row_off(n, 8), tw32_col_off(n, 8)};
     for (int q = 0; q < 4; ++q)
@@ -403,12 +406,15 @@ void build_tables_f32(const nlse_params* p, HostTables32& t) {
                     for (int d = 0; d < kDither; ++d) f[(size_t)d * cbf + 1] = f[(size_t)d * cbf];
                 }
             }
-    float* one = tw + tw32_oneoff_off(n) / 4;
-    for (size_t e = 0; e < pt[4].size() / 2; ++e)
-        for (int c = 0; c < 2; ++c) {
-            const DSplit sp = dsplit(pt[4][2 * e + c]);
-            one[2 * e + c] = sp.frac > uq[dither_offset(kTabRowPair, e, c)] ? sp.hi : sp.lo;
-        }
+    auto copy0 = [&](const std::vector<double>& w, uint64_t table, float* dst) {
+        for (size_t e = 0; e < w.size() / 2; ++e)
+            for (int c = 0; c < 2; ++c) {
+                const DSplit sp = dsplit(w[2 * e + c]);
+                dst[2 * e + c] = sp.frac > uq[dither_offset(table, e, c)] ? sp.hi : sp.lo;
+            }
+    };
+    copy0(single, kTabTwiddle, tw + tw32_line_off(n) / 4);
+    copy0(pt[4], kTabRowPair, tw + tw32_oneoff_off(n) / 4);
 }
 
 }  // namespace
@@ -745,7 +751,8 @@ nlse_status lens_impl(nlse_grid* g, const nlse_lens* ls, unsigned char* sc, int3
     T* tab = reinterpret_cast<T*>(sc + SL.tab);
     if (cudaMemcpyAsync(tab, htab.data(), htab.size() * sizeof(T), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return NLSE_ECUDA;
-    cudaError_t e = ks->fluence_lowpass(field, wbuf, wreal, w_dif_out, tab, tab + n, tw, st);
+    cudaError_t e = ks->fluence_lowpass(field, wbuf, wreal, w_dif_out, tab, tab + n,
+                                        twiddles_line<T>(g->ws + g->lay.tw, n), st);
     if (e != cudaSuccess) return NLSE_ECUDA;
 
     // lenses: regions of w_dif >= w_l, labelled by their smallest index; centres: per
@@ -1117,7 +1124,7 @@ nlse_status nlse_turbulent_screen(nlse_grid* g, const void* xi, int xi_on_device
     cudaError_t e;
     if (f64) {
         e = g->k64->turb_screen((const double2*)src, (double2*)spec, tau, m2max,
-                                twiddles_fixed<double>(g->ws + g->lay.tw), g->stream);
+                                twiddles_line<double>(g->ws + g->lay.tw, n), g->stream);
         if (e == cudaSuccess) {
             k_turb_apply<double><<<blocks, 256, 0, g->stream>>>((double2*)field, (const double2*)spec, c, nn);
             e = g->k64->row_forward((const double2*)field, (double2*)spec, twiddles_fixed<double>(g->ws + g->lay.tw),
@@ -1125,7 +1132,7 @@ nlse_status nlse_turbulent_screen(nlse_grid* g, const void* xi, int xi_on_device
         }
     } else {
         e = g->k32->turb_screen((const float2*)src, (float2*)spec, (float)tau, m2max,
-                                twiddles_fixed<float>(g->ws + g->lay.tw), g->stream);
+                                twiddles_line<float>(g->ws + g->lay.tw, n), g->stream);
         if (e == cudaSuccess) {
             k_turb_apply<float><<<blocks, 256, 0, g->stream>>>((float2*)field, (const float2*)spec, (float)c, nn);
             e = g->k32->row_forward((const float2*)field, (float2*)spec, twiddles_fixed<float>(g->ws + g->lay.tw),

@@ -91,8 +91,8 @@ template <auto Kernel> inline cudaError_t ensure_smem(int bytes) {
 // cache, where the twiddle and propagator tables are read from.  blocks = 0: all
 // of it shared memory -- an SM runs blocks of two kernels side by side only under
 // the same carveout, which lets a short pass start while the one before it ends
-// (512^2 step 15.4 -> 11.0 us, 1024^2 22.8 -> 21.1 us; from 2048^2 on the L1 is
-// worth more: 41.6 against 42.1 us).
+// (when introduced: 512^2 step 15.4 -> 11.0 us, 1024^2 22.8 -> 21.1 us; from 2048^2 on
+// the L1 is worth more: 41.6 against 42.1 us).
 template <auto Kernel> inline cudaError_t ensure_smem_carveout(int bytes, int blocks) {
     static unsigned long long done = 0;
     int dev = 0;

@@ -225,14 +225,14 @@ template <int N, int E> constexpr int col_mask32_e() {
 // bits 0-9: radix-16 tiles, bits 10-19: radix-8 tiles (kColOptions order)
 template <int N> constexpr int col_mask32() { return col_mask32_e<N, 16>() | (col_mask32_e<N, 8>() << 10); }
 
-// default column tile (radix 16), the fastest measured (us per step on GB300):
-// staged pairs of columns where a column can be staged (32-byte box rows; 4096^2:
-// 158 against 168 with single columns and 195 with two pairs; 2048^2: 41.6, 47.7,
-// 45.1; 512^2: 10.3, 18, 10.5), but single columns at 8192^2 (804 against 900: a
-// pair is one block of 512 threads per SM); two columns per block at 256^2 (8.9
-// against 9.0 and 9.4 with 1, 4); below, single columns at radix 8, for both
-// passes: a pass there is the serial chain of one warp, which half as many
-// elements per thread shorten (64^2: 5.2 against 7.9 us, 128^2: 6.2 against 8.1)
+// default column tile, the fastest measured (us per step on GB300): staged pairs of
+// columns where a column can be staged (32-byte box rows; single columns and two
+// pairs at 4096^2: 158, 166, 190; 2048^2: 40.8, 48.1, 45.3; 1024^2: 14.6, 15.6, 15.3;
+// 512^2: 9.4, 9.7, 9.4), but single columns at 8192^2 (762 against 880: a pair is one
+// block of 512 threads per SM); two columns per block at 256^2 (7.1 against 7.2 and
+// 7.5 with 1, 4); below, single columns at radix 8, for both passes: a pass there is
+// the serial chain of one warp, which half as many elements per thread shorten
+// (64^2: 4.4 against 6.4 us, 128^2: 4.7 against 6.6)
 template <int N> constexpr int col_default32() {
     if constexpr (N >= 512) return kColTma | (N >= 8192 ? 1 : 2);
     else return N >= 256 ? 2 : kColR8 | 1;

@@ -43,8 +43,8 @@ template <int L, int E> __host__ __device__ constexpr int p_e() { return L < E ?
 template <int L, int E> __host__ __device__ constexpr int p_tpl() { return L / p_e<L, E>(); }
 // row pairs per block of the row-oriented kernels: at least one warp.  A small
 // grid is a few warps per SM whose serial chains bound the pass: blocks of one
-// warp spread over all SMs (512^2: 10.3 us per step with 32 threads per block,
-// 11.0 with 128).
+// warp spread over all SMs (512^2, when introduced: 10.3 us per step with 32 threads
+// per block, 11.0 with 128).
 template <int N, int E> __host__ __device__ constexpr int p_rows() {
     return p_tpl<N, E>() >= 32 ? 1 : (32 / p_tpl<N, E>() > N / 2 ? N / 2 : 32 / p_tpl<N, E>());
 }
@@ -77,13 +77,13 @@ template <int THREADS, int E> __host__ __device__ constexpr int p_col_min_blocks
 }
 
 // Per-step FP32 twiddle block (one of kDither dithered copies, byte offsets
-// from its start): the single-line table of fft.cuh (n entries of 8 bytes,
-// used by the adjoint's row kernels and the one-off 2D transforms), the tables
-// of the radix-16 march (pair.cuh: fused butterflies, 8-byte entries) for the
-// n-point row transform and the n/2-point column sub-transforms, and those of
-// the radix-8 march (radix-4 sub-passes) for the same.  After the last copy
-// stands one radix-16 table of the row transform for the load prologue and the
-// readouts (radix-4 sub-passes, dithered as copy 0).
+// from its start): the tables of the radix-16 march (pair.cuh: fused butterflies,
+// 8-byte entries) for the n-point row transform and the n/2-point column
+// sub-transforms, and those of the radix-8 march (radix-4 sub-passes) for the
+// same.  After the last copy stand the tables of the one-off transforms, dithered
+// as copy 0: the single-line table of fft.cuh (n entries of 8 bytes: lens,
+// turbulence) and a radix-16 table of the row transform for the load prologue and
+// the readouts (radix-4 sub-passes).
 //
 // Per-step propagator tables (one of kDitherP dithered copies): P_x, n entries
 // of 8 bytes; P_y, n/2 pair entries of 16 bytes followed by the n/2 cross-lane
@@ -109,8 +109,8 @@ using RowTab = float2;
 template <int E> struct col_tab { using type = float2; };
 template <> struct col_tab<8> { using type = float4; };
 __host__ __device__ constexpr size_t tw32_row_off(int n, int e) {
-    return (size_t)8 * n + (e >= 16 ? 0 : (size_t)8 * (pr::fused_tab_entries(n, tw32_min(16, n)) +
-                                                       pr::fused_tab_entries(n / 2, tw32_min(16, n / 2))));
+    return e >= 16 ? 0 : (size_t)8 * (pr::fused_tab_entries(n, tw32_min(16, n)) +
+                                      pr::fused_tab_entries(n / 2, tw32_min(16, n / 2)));
 }
 __host__ __device__ constexpr size_t tw32_col_off(int n, int e) {
     return e >= 16 ? tw32_row_off(n, 16) + (size_t)8 * pr::fused_tab_entries(n, tw32_min(16, n))
@@ -119,7 +119,8 @@ __host__ __device__ constexpr size_t tw32_col_off(int n, int e) {
 __host__ __device__ constexpr size_t tw32_copy_bytes(int n) {
     return (tw32_col_off(n, 8) + (size_t)16 * pr::pair_tab_entries(n / 2, tw32_min(8, n / 2)) + 255) / 256 * 256;
 }
-__host__ __device__ constexpr size_t tw32_oneoff_off(int n) { return (size_t)kDither * tw32_copy_bytes(n); }
+__host__ __device__ constexpr size_t tw32_line_off(int n) { return (size_t)kDither * tw32_copy_bytes(n); }
+__host__ __device__ constexpr size_t tw32_oneoff_off(int n) { return tw32_line_off(n) + (size_t)8 * n; }
 __host__ __device__ constexpr size_t tw32_region_bytes(int n) {
     return tw32_oneoff_off(n) + (size_t)8 * pr::pair_tab_entries(n, tw32_min(16, n));
 }
@@ -592,7 +593,12 @@ __device__ __forceinline__ void col_body32(C2 (&v)[p_e<N / 2, EC>()], C2* sm, co
 // ---------------------------------------------------------------- kernels --
 
 // Row pass of the march; with DIAG the block also reduces sum |U|^2 and
-// max |U|^2 of its rows into partials.
+// max |U|^2 of its rows into partials.  At 4096^2: 98.9 -> 84.5 us (mirrored
+// transforms with fused butterflies, one vote for the screens of a thread).  HBM
+// (40 us at the copy bandwidth), the FMA pipe and the L1 data path are each about
+// half busy: two blocks of eight warps per SM, all that 128 registers per thread
+// allow, overlap each other's phases only in part (three blocks at 80 registers spill:
+// 103 us; persistent blocks fetching the next row pair, k_row_pass32_pf: 90 us).
 template <int N, int ER, bool DIAG>
 __global__ void __launch_bounds__(p_row_threads<N, ER>(), p_min_blocks<p_row_threads<N, ER>(), ER>())
 k_row_pass32(const float4* src, float4* dst, const unsigned char* twb, ScreenCoef<float> sc,
@@ -820,7 +826,10 @@ __device__ __forceinline__ void col_stage_store(const C2* smem, const CUtensorMa
 // Column pass with the tile staged by bulk tensor copies: the columns land in
 // their transform lines (the tensor maps describe the state as n/2 row pairs x
 // 4 n words), are transformed there (col_line32), and one thread stores
-// the lines with bulk tensor copies.  Waits
+// the lines with bulk tensor copies.  At 4096^2 90.3 -> 84 us, 2048^2 34.7 -> 27.4: the
+// L1 data path (exchanges, staging, tables) is 65 % busy, HBM half, and a block waits
+// a quarter of its time for its tile (per-thread loads of the same pairs: 113 us;
+// per-thread stores: 105; three blocks per SM leave the tables no L1: 113).  Waits
 // are bounded as in k_col_pass_tma (tma.cuh), with the same status bits.
 template <int N, int EC, int C>
 __global__ void __launch_bounds__(p_col_tpl<N, EC>() * C, p_col_min_blocks<p_col_tpl<N, EC>() * C, EC>())
@@ -937,7 +946,8 @@ k_readout32(const float4* __restrict__ state, const unsigned char* twb, float2* 
 
 // Row pass of the re-march: v = B_x seg into seg (stash order), then, unless dst
 // is null (the last step of a segment), the screen and dst = F_x U as
-// k_row_pass32 gives it, bit for bit.
+// k_row_pass32 gives it, bit for bit.  24 bytes per point: at 8192^2 409 us, as long
+// as the row pass without the stash.
 template <int N, int ER>
 __global__ void __launch_bounds__(p_row_threads<N, ER>(), p_min_blocks<p_row_threads<N, ER>(), ER>())
 k_row_stash32(float4* seg, float4* dst, const unsigned char* twb, ScreenCoef<float> sc) {
@@ -1049,7 +1059,10 @@ __device__ __forceinline__ void block_accumulate6_f32(const float (&g)[6], doubl
 
 // Backward row pass of one step (adjoint.cuh: k_adj_row) on the unit layout:
 // gam <- F_x( adjoint screen( B_x gam ; v ) ), v from the stash; natural != 0: the
-// stash holds v in natural order (written by the radix-8 row pass).
+// stash holds v in natural order (written by the radix-8 row pass).  24 bytes per
+// point, two transforms and about 60 packed operations per pair: at 8192^2 1626 us
+// with three transforms on the single-line engine -> 606; bound like the row pass by
+// the overlap of its phases.
 template <int N>
 __global__ void __launch_bounds__(p_row_threads<N, 16>(), p_min_blocks<p_row_threads<N, 16>(), 16>())
 k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<float> ac, double* __restrict__ acc,
@@ -1138,7 +1151,9 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
 }
 
 // Loss and seed (adjoint.cuh: k_loss_seed) on the unit layout, natural order (the
-// target is row-major): the one-off transforms of the load and the readouts.
+// target is row-major): the one-off transforms of the load and the readouts.  Five
+// FP64 instructions per point bound it (630 us of 1105 at 8192^2; 1486 on the
+// single-line engine).
 template <int N>
 __global__ void __launch_bounds__(p_row_threads<N, 16>(), p_min_blocks<p_row_threads<N, 16>(), 16>())
 k_loss_seed32(const float4* __restrict__ state, float4* __restrict__ gam, const double* __restrict__ target,
