@@ -6,7 +6,8 @@ SM of the persistent batched launch (per size mix).  Each candidate is timed on
 the GPU with CUDA events; the fastest is cached in a JSON file
 (NLSE_TUNE_CACHE, default ~/.cache/paper_2306_15678_gb300/tune.json).  For a
 given radix the results do not depend on the tile, bit for bit; the radix
-changes the rounding within the stated tolerances."""
+changes the rounding within the stated tolerances.  The keys carry a version of
+the kernels: choices timed on earlier ones are not taken up."""
 from __future__ import annotations
 
 import collections
@@ -71,7 +72,7 @@ def tune_launch(cfg: dict, precision: str = "fp32", steps: int = 20, path: str |
     then the row radices with the chosen tile."""
     path = path or cache_path()
     cache = _load_cache(path)
-    key = f"{_gpu_key()}|launch2|{precision}|{int(cfg['n'])}"
+    key = f"{_gpu_key()}|launch3|{precision}|{int(cfg['n'])}"
     if key in cache and not force:
         return {"cols": int(cache[key]["cols"]), "row_radix": int(cache[key]["row_radix"])}
     U0 = beams.make_field(cfg)
@@ -123,7 +124,7 @@ def tune_batch(cfgs: list, steps: int = 10, path: str | None = None, force: bool
     path = path or cache_path()
     cache = _load_cache(path)
     mix = collections.Counter(int(c["n"]) for c in cfgs)
-    key = f"{_gpu_key()}|batch3|" + ",".join(f"{n}x{mix[n]}" for n in sorted(mix))
+    key = f"{_gpu_key()}|batch4|" + ",".join(f"{n}x{mix[n]}" for n in sorted(mix))
     if key in cache and not force:
         return dict(cache[key]["tuning"])
     fields = fields or [beams.make_field(c).astype(np.complex64) for c in cfgs]
