@@ -300,26 +300,8 @@ template <int R, bool INV, typename V> __device__ __forceinline__ void dft(V (&a
         // 8 = 2 x 4: even/odd DFT4 then combine with W_8^k = W_16^(2k)
         dft4<INV>(a[0], a[2], a[4], a[6]);
         dft4<INV>(a[1], a[3], a[5], a[7]);
-        V e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6];
-        if constexpr (std::is_same<V, double2>::value) {
-            // products by r2 (1 - i) and r2 (-1 - i) (conjugates: INV) fused with the
-            // sums: 4 FP64 instructions fewer, one rounding fewer on each result
-            constexpr double r2 = 0.70710678118654752440;
-            const V x1 = a[3], o2 = rot4<INV>(a[5]), x3 = a[7], z = a[1];
-            const double s1 = x1.x + x1.y, d1 = x1.y - x1.x, s3 = x3.x + x3.y, d3 = x3.y - x3.x;
-            // W^1 x1 = r2 (s1, d1), inverse r2 (-d1, s1); W^3 x3 = r2 (d3, -s3), inverse r2 (-s3, -d3)
-            const double p1 = INV ? -d1 : s1, q1 = INV ? s1 : d1, p3 = INV ? -s3 : d3, q3 = INV ? -d3 : -s3;
-            a[0] = cadd(e0, z);
-            a[4] = csub(e0, z);
-            a[1] = mk<V>(fma(r2, p1, e1.x), fma(r2, q1, e1.y));
-            a[5] = mk<V>(fma(-r2, p1, e1.x), fma(-r2, q1, e1.y));
-            a[2] = cadd(e2, o2);
-            a[6] = csub(e2, o2);
-            a[3] = mk<V>(fma(r2, p3, e3.x), fma(r2, q3, e3.y));
-            a[7] = mk<V>(fma(-r2, p3, e3.x), fma(-r2, q3, e3.y));
-            return;
-        }
         V o1 = w16f<2, INV>(a[3]), o2 = w16f<4, INV>(a[5]), o3 = w16f<6, INV>(a[7]);
+        V e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6];
         a[0] = cadd(e0, a[1]); a[4] = csub(e0, a[1]);
         a[1] = cadd(e1, o1);   a[5] = csub(e1, o1);
         a[2] = cadd(e2, o2);   a[6] = csub(e2, o2);
