@@ -1,12 +1,14 @@
-"""The branches of the screens and of the launch rules that the sizes and
-intensities of a call choose between, each at the edges where it takes over,
-against the same step in FP64 numpy or the FP64 oracle."""
+"""The branches that the sizes, intensities, launch shapes and pointers of a call
+choose between, each at the edges where it takes over, against the same
+operation in FP64 numpy or its other branch."""
 import math
 
 import numpy as np
 import pytest
+import torch
 
-from paper_2306_15678_gb300 import configs
+from paper_2306_15678_gb300 import beams, capi, configs
+from paper_2306_15678_gb300.adjoint import AdjointMarch
 from paper_2306_15678_gb300.grid import Grid
 
 pytestmark = pytest.mark.gpu
@@ -80,3 +82,66 @@ def test_screen_forms(n, K, exact):
             tol = base + (abs(aK) * umax + K * abs(aP) * umax ** K) * eps
             err = np.linalg.norm(got - ref) / np.linalg.norm(ref)
             assert err < tol, (umax, prec, err, tol)
+
+
+@pytest.mark.parametrize("n", [8, 64, 512, 1024])
+def test_adjoint_stash_orders(n):
+    """The re-march leaves the fields in the order of its row pass's threads: natural
+    for radix 8, permuted for radix 16 from 512 points on.  Both give the gradients
+    of the FP64 adjoint to the scope's 1e-3 (a wrong order is an O(1) error)."""
+    cfg = configs.physics(n, 8.0, 1.0, configs.ALL_TERMS, (1.1, 0.02, 1.0, 0.0, 1.0, 0.0))
+    beam = dict(w0=1.0, P=50.0 * configs.critical_power(), amp=0.05, ell_cells=2.0, phase=0.1)
+    U = beams.make_field(dict(cfg, beam=dict(beam, seed=3, phase_seed=4)))
+    D = np.abs(beams.make_field(dict(cfg, beam=dict(beam, w0=1.1, seed=5, phase_seed=6)))) ** 2
+    got = []
+    for prec, launch in (("fp64", None), ("fp32", {"cols": 1, "row_radix": 16}),
+                         ("fp32", {"cols": capi.NLSE_COL_R8 | 1, "row_radix": 8})):
+        fit = AdjointMarch(cfg, 5, 2, precision=prec)
+        if launch:
+            fit.set_launch(launch)
+        fit.set_target(D)
+        loss = fit.forward(U)
+        dth, dU = fit.backward()
+        got.append((loss, dth, dU.cpu().numpy().astype(np.complex128)))
+        fit.close()
+    ref = got[0]
+    for loss, dth, dU in got[1:]:
+        assert abs(loss / ref[0] - 1) < 1e-3
+        assert np.linalg.norm(dth - ref[1]) < 1e-3 * np.linalg.norm(ref[1])
+        assert np.linalg.norm(dU - ref[2]) < 1e-3 * np.linalg.norm(ref[2])
+
+
+@pytest.mark.parametrize("n,conn", [(8, 4), (16, 8), (64, 8), (256, 4)])
+def test_hot_area_labels_at_any_alignment(n, conn):
+    """Device labels that the 16-byte accesses cannot use give the same labels."""
+    cfg = configs.physics(n, 1.0, 0.5, configs.KERR)
+    with Grid(cfg, precision="fp32") as g:
+        g.load(noise_field(n, 1.0, n).astype(np.complex64))
+        count, ref = g.hot_areas(0.55 * IREF, conn, labels=True)
+        buf = torch.full((n * n + 8,), -7, dtype=torch.int32, device="cuda")
+        for off in (0, 1, 2, 3):
+            buf.fill_(-7)
+            assert capi.nlse_hot_areas(g.h, 0.55 * IREF, conn, buf.data_ptr() + 4 * off, True) == count
+            out = buf.cpu().numpy()
+            assert np.array_equal(out[off:off + n * n].reshape(n, n), ref)
+            assert (out[:off] == -7).all() and (out[off + n * n:] == -7).all()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-4)])
+@pytest.mark.parametrize("n", [8, 64, 512, 2048])
+def test_moment_powers(n, prec, tol):
+    """Every kind of exponent (0, 1, 2, odd, even, the largest); positive terms, so the
+    sums follow the relative error of I^p: 16 times 2^-53 and the transforms', or
+    16 times the FP32 load and readout's 1e-6."""
+    L = 0.02 * n
+    cfg = configs.physics(n, L, 0.5, configs.KERR)
+    u = 0.5 + 0.5 * np.random.default_rng(n).random((n, n))
+    U = np.sqrt(u).astype(np.complex64).astype(np.complex128)
+    x = (np.arange(n) - n / 2 + 0.5) * (L / n)
+    r2 = x[:, None] ** 2 + x[None, :] ** 2
+    pq = [(1, 0), (1, 1), (2, 2), (3, 5), (4, 0), (7, 3), (16, 16), (6, 12)]
+    with Grid(cfg, precision=prec) as g:
+        got = g.load(U if prec == "fp64" else U.astype(np.complex64)).moments(pq)
+    for k, (p, q) in enumerate(pq):
+        ref = float((np.abs(U) ** (2 * p) * r2 ** q).sum()) * (L / n) ** 2
+        assert abs(got[k] / ref - 1) < tol, (p, q, got[k] / ref - 1)
