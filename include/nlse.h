@@ -465,13 +465,16 @@ nlse_status nlse_adjoint_set_target(nlse_adjoint* a, const double* target, int o
 
 /* March U0 (n x n interleaved complex of the grid precision, host or device)
  * M steps with checkpoints, then evaluate J (FP64) into *loss and seed the
- * adjoint.  NLSE_ESTATE without a target.  Synchronises. */
+ * adjoint.  NLSE_ESTATE without a target; NLSE_ETIMEOUT when a bounded wait of
+ * a staged pass ran out (nlse_set_column_tile): part of the field was left out,
+ * *loss is not written and there is no forward run.  Synchronises. */
 nlse_status nlse_adjoint_forward(nlse_adjoint* a, const void* U0, int on_device, double* loss);
 
 /* Backward sweep after nlse_adjoint_forward: dtheta[6] (host) receives dJ/dtheta
  * summed in FP64 in a fixed order; dU0 (n x n complex of the grid precision,
  * host or device) receives dJ/dU0.  Consumes the forward run (NLSE_ESTATE if
- * there is none).  Synchronises. */
+ * there is none).  NLSE_ETIMEOUT when a bounded wait of a staged pass ran out:
+ * dtheta is not written and dU0 is not to be used.  Synchronises. */
 nlse_status nlse_adjoint_backward(nlse_adjoint* a, double* dtheta, void* dU0, int dU0_on_device);
 
 /* Release the handle (not the workspace).  Synchronises. */

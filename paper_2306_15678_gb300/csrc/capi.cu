@@ -1267,6 +1267,14 @@ nlse_status nlse_destroy(nlse_grid* g) {
 
 namespace {
 
+// what a sweep leaves besides the sums: (loss, maximum) and the status word of its
+// passes (bit 0: non-finite, bits 1 and 2: a bounded wait ran out), which the calls
+// clear, hand to every pass and read back with their results
+struct AdjResult {
+    double value[2];
+    int status, unused;
+};
+
 struct AdjLayout {
     size_t state, gam, tw, px, py, pxc, pyc, seg, ckpt, target, partials, acc, result, total;
     int nck;
@@ -1290,8 +1298,9 @@ AdjLayout adj_layout_for(int n, int precision, int nsteps, int ckpt) {
     L.ckpt = o;     o = align256(o + field * (size_t)L.nck);
     L.target = o;   o = align256(o + (size_t)n * n * sizeof(double));
     L.partials = o; o = align256(o + (size_t)n * 2 * sizeof(double));
-    L.acc = o;      o = align256(o + (size_t)n * 6 * sizeof(double));
-    L.result = o;   o = align256(o + 4 * sizeof(double) + sizeof(int));
+    // the theta sums, then the result and the status word: one clear and one copy for all
+    L.acc = o;      o += (size_t)n * 6 * sizeof(double);
+    L.result = o;   o = align256(o + sizeof(AdjResult));
     L.total = o;
     return L;
 }
@@ -1324,6 +1333,10 @@ struct nlse_adjoint {
     AdjCoef<double> ac64;
     double sum_d2;
     int have_target, have_forward;
+    // test hooks, 0 in use: bytes that block 0 of a staged pass expects on top of its
+    // copies' (NLSE_DEBUG_COL_EXTRA_TX and NLSE_DEBUG_ROW_EXTRA_TX in the forward run,
+    // NLSE_DEBUG_ADJ_BACK_EXTRA_TX in the column passes of the backward sweep)
+    unsigned debug_col_extra_tx, debug_row_extra_tx, debug_back_extra_tx;
 };
 
 namespace {
@@ -1345,6 +1358,8 @@ template <typename T> const WT<T>* atab(nlse_adjoint* a, size_t off) {
 inline size_t adj_field_bytes(const nlse_adjoint* a) {
     return (size_t)a->p.n * a->p.n * (a->p.precision == NLSE_FP64 ? 16 : 8);
 }
+
+inline AdjResult* adj_result(nlse_adjoint* a) { return reinterpret_cast<AdjResult*>(a->ws + a->lay.result); }
 
 template <typename T> nlse_status adj_upload(nlse_adjoint* a);
 template <> nlse_status adj_upload<double>(nlse_adjoint* a) {
@@ -1393,7 +1408,9 @@ template <typename T> nlse_status adj_forward_impl(nlse_adjoint* a, const void* 
     const WT<T>* tw = twiddles_fixed<T>(a->ws + a->lay.tw);
     const int n = a->p.n;
     const size_t fb = adj_field_bytes(a);
-    cudaError_t e;
+    AdjResult* result = adj_result(a);
+    cudaError_t e = cudaMemsetAsync(result, 0, sizeof(AdjResult), a->stream);
+    if (e != cudaSuccess) return NLSE_ECUDA;
     if (on_device) {
         e = ks->row_forward((const VT<T>*)src, state, tw, a->stream);
     } else {  // the host field is staged in gam (free until the backward sweep)
@@ -1411,26 +1428,25 @@ template <typename T> nlse_status adj_forward_impl(nlse_adjoint* a, const void* 
             return NLSE_ECUDA;
         const WT<T>* tws = twiddles_at<T>(a->ws + a->lay.tw, n, s);
         if (ks->col_pass(state, state, tws, px_at<T>(a->ws + a->lay.px, n, s),
-                         py_at<T>(a->ws + a->lay.py, n, s), rot_for_step<T>(s, nullptr), a->cols, nullptr,
-                         0u, a->stream) != cudaSuccess)
+                         py_at<T>(a->ws + a->lay.py, n, s), rot_for_step<T>(s, nullptr), a->cols, &result->status,
+                         a->debug_col_extra_tx, a->stream) != cudaSuccess)
             return NLSE_ECUDA;
-        if (ks->row_pass(state, state, tws, sc, partials, false, a->row_radix, nullptr, 0u, a->stream) !=
-            cudaSuccess)
+        if (ks->row_pass(state, state, tws, sc, partials, false, a->row_radix, &result->status,
+                         a->debug_row_extra_tx, a->stream) != cudaSuccess)
             return NLSE_ECUDA;
     }
-    double* result = reinterpret_cast<double*>(a->ws + a->lay.result);
     if (ks->loss_seed(state, aat<T>(a, a->lay.gam), reinterpret_cast<const double*>(a->ws + a->lay.target),
                       tw, 1.0 / a->sum_d2, partials, a->stream) != cudaSuccess)
         return NLSE_ECUDA;
-    k_finalize<<<1, 256, 0, a->stream>>>(partials, ks->adj_blocks, 1.0 / a->sum_d2, result,
-                                         reinterpret_cast<int*>(result + 4));
+    k_finalize<<<1, 256, 0, a->stream>>>(partials, ks->adj_blocks, 1.0 / a->sum_d2, result->value, &result->status);
     if (cudaGetLastError() != cudaSuccess) return NLSE_ECUDA;
-    double r[2];
-    if (cudaMemcpyAsync(r, result, sizeof(r), cudaMemcpyDeviceToHost, a->stream) != cudaSuccess)
+    AdjResult r;
+    if (cudaMemcpyAsync(&r, result, sizeof(r), cudaMemcpyDeviceToHost, a->stream) != cudaSuccess)
         return NLSE_ECUDA;
     if (cudaStreamSynchronize(a->stream) != cudaSuccess) return NLSE_ECUDA;
-    *loss = r[0];
-    return std::isfinite(r[0]) ? NLSE_OK : NLSE_ENONFINITE;
+    if (r.status & 6) return NLSE_ETIMEOUT;  // a pass left out part of the field
+    *loss = r.value[0];
+    return std::isfinite(r.value[0]) ? NLSE_OK : NLSE_ENONFINITE;
 }
 
 template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dtheta, void* dU0, int on_device) {
@@ -1443,7 +1459,9 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
     const size_t fb = adj_field_bytes(a);
     double* partials = reinterpret_cast<double*>(a->ws + a->lay.partials);
     double* acc = reinterpret_cast<double*>(a->ws + a->lay.acc);
-    if (cudaMemsetAsync(acc, 0, (size_t)a->p.n * 6 * sizeof(double), a->stream) != cudaSuccess)
+    int* status = &adj_result(a)->status;
+    const size_t sums = (size_t)a->p.n * 6;
+    if (cudaMemsetAsync(acc, 0, sums * sizeof(double) + sizeof(AdjResult), a->stream) != cudaSuccess)
         return NLSE_ECUDA;
     auto seg = [&](int i) { return reinterpret_cast<VT<T>*>(a->ws + a->lay.seg + fb * (size_t)i); };
     for (int c = (a->nsteps - 1) / a->ckpt; c >= 0; --c) {
@@ -1456,13 +1474,13 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
             const bool last = s + 1 == c1;
             if (ks->col_pass(state, seg(s - c0), tws, px_at<T>(a->ws + a->lay.px, n, s),
                              py_at<T>(a->ws + a->lay.py, n, s), rot_for_step<T>(s, nullptr), a->cols,
-                             nullptr, 0u, a->stream) != cudaSuccess)
+                             status, a->debug_back_extra_tx, a->stream) != cudaSuccess)
                 return NLSE_ECUDA;
             if (ks->row_stash) {
                 if (ks->row_stash(seg(s - c0), last ? nullptr : state, tws, ac.sc, a->row_radix, a->stream) !=
                     cudaSuccess)
                     return NLSE_ECUDA;
-            } else if (!last && ks->row_pass(seg(s - c0), state, tws, ac.sc, partials, false, a->row_radix, nullptr,
+            } else if (!last && ks->row_pass(seg(s - c0), state, tws, ac.sc, partials, false, a->row_radix, status,
                                              0u, a->stream) != cudaSuccess) {
                 return NLSE_ECUDA;
             }
@@ -1473,7 +1491,7 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
                 return NLSE_ECUDA;
             if (ks->col_pass(gam, gam, tws, px_at<T>(a->ws + a->lay.pxc, n, s),
                              py_at<T>(a->ws + a->lay.pyc, n, s), conj_of(rot_for_step<T>(s, nullptr)), a->cols,
-                             nullptr, 0u, a->stream) != cudaSuccess)
+                             status, a->debug_back_extra_tx, a->stream) != cudaSuccess)
                 return NLSE_ECUDA;
         }
     }
@@ -1483,7 +1501,7 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
     scale.y = (T)0;
     VT<T>* out = on_device ? (VT<T>*)dU0 : seg(0);
     if (ks->readout(gam, tw, out, nullptr, partials, scale, a->stream) != cudaSuccess) return NLSE_ECUDA;
-    std::vector<double> h((size_t)a->p.n * 6);
+    std::vector<double> h(sums + sizeof(AdjResult) / sizeof(double));
     if (cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(double), cudaMemcpyDeviceToHost, a->stream) !=
         cudaSuccess)
         return NLSE_ECUDA;
@@ -1491,6 +1509,9 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
         cudaMemcpyAsync(dU0, out, fb, cudaMemcpyDeviceToHost, a->stream) != cudaSuccess)
         return NLSE_ECUDA;
     if (cudaStreamSynchronize(a->stream) != cudaSuccess) return NLSE_ECUDA;
+    AdjResult r;
+    std::memcpy(&r, h.data() + sums, sizeof(r));
+    if (r.status & 6) return NLSE_ETIMEOUT;  // a pass left out part of the field
     for (int q = 0; q < 6; ++q) dtheta[q] = 0.0;
     for (int b = 0; b < ks->adj_blocks; ++b)  // fixed order: deterministic
         for (int q = 0; q < 6; ++q) dtheta[q] += h[6 * (size_t)b + q];
@@ -1530,6 +1551,10 @@ nlse_status nlse_adjoint_create(const nlse_params* p, int32_t nsteps, int32_t ck
     a->stream = static_cast<cudaStream_t>(cuda_stream);
     a->ws = static_cast<unsigned char*>(dev_workspace);
     a->lay = lay;
+    if (const char* env = std::getenv("NLSE_DEBUG_COL_EXTRA_TX")) a->debug_col_extra_tx = (unsigned)std::atoi(env);
+    if (const char* env = std::getenv("NLSE_DEBUG_ROW_EXTRA_TX")) a->debug_row_extra_tx = (unsigned)std::atoi(env);
+    if (const char* env = std::getenv("NLSE_DEBUG_ADJ_BACK_EXTRA_TX"))
+        a->debug_back_extra_tx = (unsigned)std::atoi(env);
     const int k = log2_exact(p->n);
     if (p->precision == NLSE_FP64) {
         a->k64 = kernels_f64(k);
@@ -1586,12 +1611,12 @@ nlse_status nlse_adjoint_set_target(nlse_adjoint* a, const double* target, int o
                         a->stream) != cudaSuccess)
         return NLSE_ECUDA;
     double* partials = reinterpret_cast<double*>(a->ws + a->lay.partials);
-    double* result = reinterpret_cast<double*>(a->ws + a->lay.result);
+    AdjResult* result = adj_result(a);
     k_sumsq_rows<<<n, 256, 0, a->stream>>>(d, n, partials);
-    k_finalize<<<1, 256, 0, a->stream>>>(partials, n, 1.0, result, reinterpret_cast<int*>(result + 4));
+    k_finalize<<<1, 256, 0, a->stream>>>(partials, n, 1.0, result->value, &result->status);
     if (cudaGetLastError() != cudaSuccess) return NLSE_ECUDA;
     double r[2];
-    if (cudaMemcpyAsync(r, result, sizeof(r), cudaMemcpyDeviceToHost, a->stream) != cudaSuccess)
+    if (cudaMemcpyAsync(r, result->value, sizeof(r), cudaMemcpyDeviceToHost, a->stream) != cudaSuccess)
         return NLSE_ECUDA;
     if (cudaStreamSynchronize(a->stream) != cudaSuccess) return NLSE_ECUDA;
     if (!(r[0] > 0.0) || !std::isfinite(r[0])) return NLSE_EINVAL;  // an all-zero target has no loss scale
