@@ -1030,20 +1030,21 @@ __device__ __forceinline__ C2 adj_value2(C2 v, C2 G, F2 u, F2 re, F2 im, F2 dre,
             fma(q, v.im, add(G.im, fma(dre, G.im, mul(neg(dim), G.re))))};
 }
 
-// Six per-thread FP32 sums -> FP64 sums added into acc[block][6], in a fixed order:
-// each warp takes sums 0..5 in turn, its lanes every 32nd thread's value, then a
-// shuffle tree.  (A tree of FP64 shuffles in every warp is 30 FP64 additions per
+// Six per-thread pairs of FP32 sums (one per row) -> FP64 sums added into
+// acc[block][6], in a fixed order: each warp takes sums 0..5 in turn, its lanes every
+// 32nd thread's pair, then a shuffle tree.  The rows of a pair are joined in FP64 like
+// all others.  (A tree of FP64 shuffles in every warp is 30 FP64 additions per
 // thread: at 8192^2 a fifth of the kernel.)
 template <int THREADS>
-__device__ __forceinline__ void block_accumulate6_f32(const float (&g)[6], double* __restrict__ acc) {
-    __shared__ float red[6][THREADS];
+__device__ __forceinline__ void block_accumulate6_f32(const F2 (&g)[6], double* __restrict__ acc) {
+    __shared__ float2 red[6][THREADS];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = g[q];
+    for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = make_float2(pr::lo(g[q]), pr::hi(g[q]));
     __syncthreads();
     if constexpr (THREADS >= 32) {
         for (int q = (int)threadIdx.x >> 5; q < 6; q += THREADS / 32) {
             double s = 0.0;
-            for (int i = (int)threadIdx.x & 31; i < THREADS; i += 32) s += (double)red[q][i];
+            for (int i = (int)threadIdx.x & 31; i < THREADS; i += 32) s += (double)red[q][i].x + (double)red[q][i].y;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if ((threadIdx.x & 31) == 0) acc[6 * blockIdx.x + q] += s;
@@ -1051,7 +1052,7 @@ __device__ __forceinline__ void block_accumulate6_f32(const float (&g)[6], doubl
     } else {
         for (int q = threadIdx.x; q < 6; q += THREADS) {
             double s = 0.0;
-            for (int i = 0; i < THREADS; ++i) s += (double)red[q][i];
+            for (int i = 0; i < THREADS; ++i) s += (double)red[q][i].x + (double)red[q][i].y;
             acc[6 * blockIdx.x + q] += s;
         }
     }
@@ -1144,10 +1145,7 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
     pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) UnitPlain::st(gam + row + j + m * T, v[m]);
-    float s6[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) s6[q] = pr::lo(th[q]) + pr::hi(th[q]);
-    block_accumulate6_f32<p_row_threads<N, 16>()>(s6, acc);
+    block_accumulate6_f32<p_row_threads<N, 16>()>(th, acc);
 }
 
 // Loss and seed (adjoint.cuh: k_loss_seed) on the unit layout, natural order (the
