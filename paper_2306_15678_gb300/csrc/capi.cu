@@ -732,7 +732,7 @@ nlse_status lens_impl(nlse_grid* g, const nlse_lens* ls, unsigned char* sc, int3
     V* field = at<T>(g, g->lay.aux);
     const auto* tw = twiddles_fixed<T>(g->ws + g->lay.tw);
     cudaStream_t st = g->stream;
-    const int blocks = (int)std::min<size_t>((nn / 4 + 255) / 256, 152 * 8);
+    const int blocks = (int)std::min<size_t>((nn + 255) / 256, 152 * 8);
 
     // the field leaves the state for the scratch half of the grid (row-major,
     // global phase removed) and comes back after the screen
@@ -760,13 +760,11 @@ nlse_status lens_impl(nlse_grid* g, const nlse_lens* ls, unsigned char* sc, int3
     const int rt = n / 4 < 256 ? n / 4 : 256;
     if constexpr (F32) k_hot_runs<T><<<n, rt, 0, st>>>(wreal, n, 1, (T)ls->w_l, lab);
     else k_hot_runs<T><<<n, rt, 0, st>>>(reinterpret_cast<const T*>(wbuf), n, 2, (T)ls->w_l, lab);
-    k_hot_merge<<<blocks, 256, 0, st>>>(lab, n, ls->connectivity, ctr + 1);
-    k_hot_roots<true><<<blocks, 256, 0, st>>>(lab, n, ctr, F32 ? list : nullptr, key, cen);
     if constexpr (F32) {
-        k_hot_spread<<<blocks, 256, 0, st>>>(lab, (int)nn, LensMax32{wreal, key});
+        hot_sweeps<true>(lab, n, ls->connectivity, ctr, ctr + 1, key, cen, LensMax32{wreal, key, list, ctr + 2}, st);
         k_lens_centres<<<32, 256, 0, st>>>(list, ctr, key);
     } else {
-        k_hot_spread<<<blocks, 256, 0, st>>>(lab, (int)nn, LensMax64{wbuf, key});
+        hot_sweeps<true>(lab, n, ls->connectivity, ctr, ctr + 1, key, cen, LensMax64{wbuf, key}, st);
         k_lens_argmax<<<blocks, 256, 0, st>>>(wbuf, lab, key, cen, nn);
         k_lens_gather<<<blocks, 256, 0, st>>>(lab, cen, list, ctr + 2, nn);  // (the keys are done with)
     }
@@ -1076,10 +1074,7 @@ nlse_status nlse_hot_areas(nlse_grid* g, double w_p, int32_t connectivity, int32
     const int rt = n / 4 < 256 ? n / 4 : 256;
     if (f64) k_hot_runs<double><<<n, rt, 0, g->stream>>>((const double*)flu, n, 1, w_p, lab);
     else k_hot_runs<float><<<n, rt, 0, g->stream>>>((const float*)flu, n, 1, (float)w_p, lab);
-    const int blocks = std::min((nn / 4 + 255) / 256, 152 * 8);
-    k_hot_merge<<<blocks, 256, 0, g->stream>>>(lab, n, connectivity, word + 1);
-    k_hot_roots<false><<<blocks, 256, 0, g->stream>>>(lab, n, word, nullptr, nullptr, nullptr);
-    k_hot_spread<<<blocks, 256, 0, g->stream>>>(lab, nn, HotNothing{});
+    hot_sweeps<false>(lab, n, connectivity, word, word + 1, nullptr, nullptr, HotNothing{}, g->stream);
     if (cudaGetLastError() != cudaSuccess) return NLSE_ECUDA;
     int host_word[2] = {0, 0};
     if (cudaMemcpyAsync(host_word, word, sizeof(host_word), cudaMemcpyDeviceToHost, g->stream) != cudaSuccess)

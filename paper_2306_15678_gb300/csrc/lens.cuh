@@ -35,12 +35,16 @@ __device__ __forceinline__ unsigned long long lens_key(double w) { return (unsig
 // What the labels' spreading sweep (hot_areas.cuh) does for each pixel of a lens:
 // key[root] = largest key (reset when the root was found).  FP32 keys carry the
 // pixel below the value, inverted, so that the largest key is the first pixel of
-// the largest value; FP64 keys fill the word, and k_lens_argmax finds the pixel.
+// the largest value, and each root appends itself to list (here, where the warps keep
+// step: the list comes out nearly sorted, and the host sorts it); FP64 keys fill the
+// word, and k_lens_argmax finds the pixel.
 struct LensMax32 {
     const float* w;
     unsigned long long* key;
+    int *list, *count;
     __device__ __forceinline__ void operator()(int root, int i) const {
         atomicMax(&key[root], (lens_key(w[i]) << 32) | (0xffffffffu - (unsigned)i));
+        if (root == i) list[atomicAdd(count, 1)] = i;
     }
 };
 struct LensMax64 {
