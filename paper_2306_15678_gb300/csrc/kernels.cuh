@@ -572,7 +572,10 @@ __device__ __forceinline__ void col_tile(const typename vec2<T>::type* src, type
         }
     }
     conj_all(v);
-    pdl_trigger();
+    // (from 512^2 on not where the tiles leave SMs without a block: the row pass's blocks
+    // would pile up there -- 512^2, 4 columns per block, 125 us per step with, 99 without;
+    // at 256^2 every tile gains from it)
+    if constexpr (N < 512 || N / C >= 152) pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) M::st(dst + sidx<N>(j + m * TL, col), v[m]);
 }
