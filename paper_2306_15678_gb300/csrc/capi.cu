@@ -1263,8 +1263,8 @@ nlse_status nlse_destroy(nlse_grid* g) {
 namespace {
 
 // what a sweep leaves besides the sums: (loss, maximum) and the status word of its
-// passes (bit 0: non-finite, bits 1 and 2: a bounded wait ran out), which the calls
-// clear, hand to every pass and read back with their results
+// passes (bit 0: non-finite, bits 1 and 2: a bounded wait ran out), which every pass
+// gets and the calls read back with their results
 struct AdjResult {
     double value[2];
     int status, unused;
@@ -1328,6 +1328,7 @@ struct nlse_adjoint {
     AdjCoef<double> ac64;
     double sum_d2;
     int have_target, have_forward;
+    int status_clear;  // bits 1 and 2 of the status word were 0 when a call last read it, and no pass ran since
     // test hooks, 0 in use: bytes that block 0 of a staged pass expects on top of its
     // copies' (NLSE_DEBUG_COL_EXTRA_TX and NLSE_DEBUG_ROW_EXTRA_TX in the forward run,
     // NLSE_DEBUG_ADJ_BACK_EXTRA_TX in the column passes of the backward sweep)
@@ -1404,8 +1405,10 @@ template <typename T> nlse_status adj_forward_impl(nlse_adjoint* a, const void* 
     const int n = a->p.n;
     const size_t fb = adj_field_bytes(a);
     AdjResult* result = adj_result(a);
-    cudaError_t e = cudaMemsetAsync(result, 0, sizeof(AdjResult), a->stream);
+    cudaError_t e = cudaSuccess;
+    if (!a->status_clear) e = cudaMemsetAsync(result, 0, sizeof(AdjResult), a->stream);
     if (e != cudaSuccess) return NLSE_ECUDA;
+    a->status_clear = 0;
     if (on_device) {
         e = ks->row_forward((const VT<T>*)src, state, tw, a->stream);
     } else {  // the host field is staged in gam (free until the backward sweep)
@@ -1440,6 +1443,7 @@ template <typename T> nlse_status adj_forward_impl(nlse_adjoint* a, const void* 
         return NLSE_ECUDA;
     if (cudaStreamSynchronize(a->stream) != cudaSuccess) return NLSE_ECUDA;
     if (r.status & 6) return NLSE_ETIMEOUT;  // a pass left out part of the field
+    a->status_clear = 1;
     *loss = r.value[0];
     return std::isfinite(r.value[0]) ? NLSE_OK : NLSE_ENONFINITE;
 }
@@ -1455,6 +1459,7 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
     double* partials = reinterpret_cast<double*>(a->ws + a->lay.partials);
     double* acc = reinterpret_cast<double*>(a->ws + a->lay.acc);
     int* status = &adj_result(a)->status;
+    a->status_clear = 0;
     const size_t sums = (size_t)a->p.n * 6;
     if (cudaMemsetAsync(acc, 0, sums * sizeof(double) + sizeof(AdjResult), a->stream) != cudaSuccess)
         return NLSE_ECUDA;
@@ -1507,6 +1512,7 @@ template <typename T> nlse_status adj_backward_impl(nlse_adjoint* a, double* dth
     AdjResult r;
     std::memcpy(&r, h.data() + sums, sizeof(r));
     if (r.status & 6) return NLSE_ETIMEOUT;  // a pass left out part of the field
+    a->status_clear = 1;
     for (int q = 0; q < 6; ++q) dtheta[q] = 0.0;
     for (int b = 0; b < ks->adj_blocks; ++b)  // fixed order: deterministic
         for (int q = 0; q < 6; ++q) dtheta[q] += h[6 * (size_t)b + q];
