@@ -170,13 +170,18 @@ __device__ __forceinline__ double2 apply_screen(double2 v, const ScreenCoef<doub
     return mk<double2>(v.x * pr - v.y * pi, v.x * pi + v.y * pr);
 }
 
+// High word of a double above every magnitude whose high word is at most h (0..0x7fffffff):
+// the next one up, and infinity's for the largest numbers, infinities and every NaN.
+__host__ __device__ constexpr int hi_word_above(int h) { return (h < 0x7fefffff ? h : 0x7fefffff) + 1; }
+
 // The screen of all of a thread's values.  FP64, K = 8 and real gains (the
 // nominal case): FP64 instructions bound these passes (GB300 issues them at 1/74
 // of the FP32 rate), and exp and sincos with their general argument reduction
 // were a third of a row pass.  The largest component of the values (found on its
 // high words, by integer operations) bounds |v|^2, so one vote tells when every
-// phase is within 1/32 rad and every gain below 2^-9: Taylor polynomials to below
-// 2^-53 of the factor's change then, applied as v + v d.
+// phase is within 1/32 rad and every gain below 2^-9 (an infinite bound fails it, so
+// threads that hold an infinity or a NaN take the general form): Taylor polynomials to
+// below 2^-53 of the factor's change then, applied as v + v d.
 template <int E> __device__ __forceinline__ void apply_screens(double2 (&v)[E], const ScreenCoef<double>& c,
                                                                unsigned warp) {
     if (c.K == 8 && c.real_gains) {  // (uniform)
@@ -184,8 +189,7 @@ template <int E> __device__ __forceinline__ void apply_screens(double2 (&v)[E], 
 #pragma unroll
         for (int m = 0; m < E; ++m)
             h = max(h, max(__double2hiint(v[m].x) & 0x7fffffff, __double2hiint(v[m].y) & 0x7fffffff));
-        // next high word up: above every component (infinity or NaN stay so)
-        const double top = __hiloint2double(h + 1, 0), u = 2.0 * top * top * c.inv_iref;
+        const double top = __hiloint2double(hi_word_above(h), 0), u = 2.0 * top * top * c.inv_iref;
         const double u2 = u * u, u4 = u2 * u2;
         const double gain = fabs(c.re_a) * (u4 * u2 * u), phase = fabs(c.im_k) * u + fabs(c.im_p) * (u4 * u4);
         if (__all_sync(warp, phase <= 0.03125 && gain <= 0.001953125)) {
