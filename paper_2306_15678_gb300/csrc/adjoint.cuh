@@ -24,7 +24,8 @@ template <typename T> struct AdjCoef {
     T aK, aP, aA;
 };
 
-// (1 + d) = e^s as applied by the forward screen, and s'(I) = ds/dI
+// e^s as applied by the forward screen, and s'(I) = ds/dI (FP64; FP32: pass32.cuh,
+// adj_value2)
 template <typename T>
 __device__ __forceinline__ void screen_factor_and_slope(T u, const AdjCoef<T>& a, T* er, T* ei,
                                                         T* sr, T* si, T* uk, T* uk1) {
@@ -47,20 +48,11 @@ __device__ __forceinline__ void screen_factor_and_slope(T u, const AdjCoef<T>& a
     *si = (c.im_k + Kf * c.im_p * k1 + K1f * c.im_a * k2) * c.inv_iref;
     *uk = k;
     *uk1 = k1;
-    if constexpr (sizeof(T) == 4) {
-        const unsigned warp = (blockDim.x & 31) == 0 ? 0xffffffffu : __activemask();
-        const float em1 = c.has_gain ? expm1_(re, warp) : 0.0f;
-        float sn, cm1;
-        sin_cosm1(im, &sn, &cm1, warp);
-        *er = 1.0f + fmaf(em1, cm1, em1 + cm1);
-        *ei = fmaf(em1, sn, sn);
-    } else {
-        const double amp = exp(re);
-        double sn, cs;
-        sincos(im, &sn, &cs);
-        *er = amp * cs;
-        *ei = amp * sn;
-    }
+    const double amp = exp(re);
+    double sn, cs;
+    sincos(im, &sn, &cs);
+    *er = amp * cs;
+    *ei = amp * sn;
 }
 
 // six per-thread partial sums -> per-block FP64 sums added into acc[block][6]

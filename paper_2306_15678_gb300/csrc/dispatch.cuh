@@ -186,12 +186,9 @@ cudaError_t launch_col_c(const typename vec2<T>::type* src, typename vec2<T>::ty
     }
 }
 
-// Tensor map of an n x n complex state (state layout, see sidx) as n/2 row
-// pairs x n columns x 4 words (4-byte words for complex64, 8-byte for
-// complex128: the copies move bits, no conversion), boxes of 4 words x C
-// columns x 256 row pairs.  cuTensorMapEncodeTiled is a host-only driver call,
-// reached through the runtime's entry-point query so that the library needs no
-// link to libcuda.
+// Tensor map over `word_bytes` words (4 or 8; the copies move bits, no conversion).
+// cuTensorMapEncodeTiled is a host-only driver call, reached through the runtime's
+// entry-point query so that the library needs no link to libcuda.
 inline cudaError_t encode_map(CUtensorMap* map, const void* base, int word_bytes, const cuuint64_t (&dims)[3],
                               const cuuint64_t (&strides)[2], const cuuint32_t (&box)[3]) {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
@@ -212,12 +209,14 @@ inline cudaError_t encode_map(CUtensorMap* map, const void* base, int word_bytes
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-inline cudaError_t encode_field_map(CUtensorMap* map, const void* base, int n, int word_bytes, int cols) {
-    const cuuint64_t w = (cuuint64_t)4 * word_bytes;
-    return encode_map(map, base, word_bytes, {4, (cuuint64_t)n, (cuuint64_t)n / 2}, {w, w * n},
+// Tensor map of an n x n complex128 state (state layout, see sidx) as n/2 row pairs x
+// n columns x 4 words, boxes of 4 words x C columns x 256 row pairs.
+inline cudaError_t encode_field_map(CUtensorMap* map, const void* base, int n, int cols) {
+    const cuuint64_t w = 4 * sizeof(double);
+    return encode_map(map, base, (int)sizeof(double), {4, (cuuint64_t)n, (cuuint64_t)n / 2}, {w, w * n},
                       {4, (cuuint32_t)cols, (cuuint32_t)kTmaBoxRows});
 }
-// The same field of 16-byte FP32 units as n/2 row pairs x 4 n words: a box of
+// An n x n FP32 state of 16-byte units as n/2 row pairs x 4 n words: a box of
 // `cols` columns x box_rows row pairs is rows of 16 cols contiguous bytes
 // (the word coordinate of column c is 4 c: 16-byte aligned).
 inline cudaError_t encode_unit_map(CUtensorMap* map, const void* base, int n, int cols, int box_rows) {
@@ -234,10 +233,10 @@ cudaError_t launch_col_tma_c(const typename vec2<T>::type* src, typename vec2<T>
     if constexpr (col_valid<T, N, C>() && col_tma_valid<T, N, C>()) {
         constexpr int SMEM = col_smem_bytes<T, N, C>() + kTmaAlignPad;
         CUtensorMap ml, ms;
-        cudaError_t e = encode_field_map(&ml, src, N, (int)sizeof(T), C);
+        cudaError_t e = encode_field_map(&ml, src, N, C);
         if (e == cudaSuccess) {
             if (static_cast<const void*>(src) == static_cast<const void*>(dst)) ms = ml;
-            else e = encode_field_map(&ms, dst, N, (int)sizeof(T), C);
+            else e = encode_field_map(&ms, dst, N, C);
         }
         if (e == cudaSuccess) e = ensure_smem<k_col_pass_tma<T, N, C>>(SMEM);
         if (e != cudaSuccess) return e;

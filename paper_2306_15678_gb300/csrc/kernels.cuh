@@ -35,7 +35,8 @@ template <typename T> struct ScreenCoef {
                    // frozen screen; its absorption number is a = ka u^(K-1)
     T ka;          // (K-1) c_A beta_K dz I_ref^(K-1)
     int real_gains;  // 1: re_k = re_p = 0 and im_a = 0 (real gains, e.g. the nominal
-                     // ones): the exponent's zero terms are skipped (same values)
+                     // ones).  With K = 8 the screens take short forms of their own; FP32
+                     // also skips the exponent's zero terms value by value (same values)
     // power series in a of the exact substep (FP32, |a| <= 2^-7), coefficients of
     // a^1..a^4 of amp - 1, f1 - 1 and fk - 1 (see apply_screen_exact)
     T ex_amp[4], ex_f1[4], ex_fk[4];
@@ -130,32 +131,6 @@ template <typename T> __device__ __forceinline__ void screen_exponent(T u, const
     }
     *re = c.re_k * u + c.re_p * uk + c.re_a * uk1;
     *im = c.im_k * u + c.im_p * uk + c.im_a * uk1;
-}
-
-// FP32: U = v + v d with d = exp(re + i im) - 1 = expm1(re) e^{i im} + (e^{i im} - 1),
-// so that the per-step change, not the field, carries the rounding of the factor
-__device__ __forceinline__ float2 apply_screen(float2 v, const ScreenCoef<float>& c, unsigned warp) {
-    const float u = (v.x * v.x + v.y * v.y) * c.inv_iref;
-    float re, im;
-    screen_exponent(u, c, &re, &im);
-    // one vote for both fast paths: the usual case, every lane's phase within
-    // pi/4 and gain below 1/16 (the same bits as the general paths give)
-    float em1, sn, cm1;
-    if (__all_sync(warp, fabsf(im) <= 0.7853982f && fabsf(re) < 0.0625f)) {
-        em1 = c.has_gain ? expm1_core(re) : 0.0f;  // uniform: pure phase screens skip it
-        sin_cosm1_core(im, &sn, &cm1);
-    } else {
-        em1 = c.has_gain ? expm1_(re, warp) : 0.0f;
-        sin_cosm1(im, &sn, &cm1, warp);
-    }
-    const float dre = fmaf(em1, cm1, em1 + cm1);  // (1 + em1)(1 + cm1) - 1
-    const float dim = fmaf(em1, sn, sn);          // (1 + em1) sin
-    // the whole change v d first (accurate relative to itself), then a single
-    // rounding of v + v d: adding the small second-order part after rounding the
-    // first-order part would lose it at every step, coherently
-    const float ddx = fmaf(v.x, dre, -v.y * dim);
-    const float ddy = fmaf(v.x, dim, v.y * dre);
-    return cadd(v, mk<float2>(ddx, ddy));
 }
 
 // FP64: the factor exp(re) (cos im + i sin im) directly
@@ -471,27 +446,10 @@ template <int TL, int RPB> __device__ __forceinline__ int lane_in_row() {
     else return (int)(threadIdx.x % TL);
 }
 
-// Global-memory access policies of the tile bodies: plain accesses for the
-// per-pass kernels, L2-only (.cg) accesses for the persistent batched kernel,
-// whose tiles are rewritten by other SMs within the same launch.
-// kExactScreen: whether the body carries the exact pointwise substep (the
-// batched march takes the frozen screen only, and its persistent kernel keeps
-// the registers the substep's call would cost).
-struct MemPlain {
-    static constexpr bool kExactScreen = true;
-    template <typename V> __device__ __forceinline__ static V ld(const V* p) { return *p; }
-    template <typename V> __device__ __forceinline__ static void st(V* p, V v) { *p = v; }
-};
-struct MemCG {
-    static constexpr bool kExactScreen = false;
-    template <typename V> __device__ __forceinline__ static V ld(const V* p) { return __ldcg(p); }
-    template <typename V> __device__ __forceinline__ static void st(V* p, V v) { __stcg(p, v); }
-};
-
 // Row pass body for RPB consecutive rows starting at row0 (thread layout:
 // row group g = tid / TL, in-row index j = tid % TL): v = B_x S, screen,
 // S = F_x U.  With DIAG, adds the thread's sum and max of |U|^2.
-template <typename T, int N, int RPB, bool DIAG, class M>
+template <typename T, int N, int RPB, bool DIAG>
 __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
                                          const typename tab_of<T>::type* __restrict__ tw,
                                          const ScreenCoef<T>& sc, int row0, typename vec2<T>::type* smem,
@@ -504,7 +462,7 @@ __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, type
     V* sm = smem + g * LS;
     V v[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = M::ld(src + sidx<N>(row, j + m * TL));
+    for (int m = 0; m < E; ++m) v[m] = src[sidx<N>(row, j + m * TL)];
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
         if (half == 0) conj_all(v);
@@ -520,7 +478,7 @@ __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, type
 #pragma unroll 1
             for (int rep = 0; rep < sc.reps; ++rep) {
                 if (sc.active) {
-                    if (M::kExactScreen && sc.exact) {  // (uniform)
+                    if (sc.exact) {  // (uniform)
 #pragma unroll
                         for (int m = 0; m < E; ++m)
                             v[m] = apply_screen_exact<T>(v[m], sc.inv_iref, sc.im_k, sc.im_p, sc.ka, sc.K);
@@ -541,7 +499,7 @@ __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, type
     }
     pdl_trigger();
 #pragma unroll
-    for (int m = 0; m < E; ++m) M::st(dst + sidx<N>(row, j + m * TL), v[m]);
+    for (int m = 0; m < E; ++m) dst[sidx<N>(row, j + m * TL)] = v[m];
 }
 
 // Column pass body for C consecutive columns starting at col0 (thread layout:
@@ -549,7 +507,7 @@ __device__ __forceinline__ void row_tile(const typename vec2<T>::type* src, type
 // S <- B_y(P_x(kx) P_y(ky) rot F_y S), P_y carrying 1/n^2 and rot = exp(i theta)
 // this step's global phase (see the march in the host code: it decorrelates
 // the FP32 rounding of the slowly rotating spectral values from step to step).
-template <typename T, int N, int C, class M>
+template <typename T, int N, int C>
 __device__ __forceinline__ void col_tile(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
                                          const typename tab_of<T>::type* __restrict__ tw,
                                          const typename tab_of<T>::type* __restrict__ px,
@@ -564,7 +522,7 @@ __device__ __forceinline__ void col_tile(const typename vec2<T>::type* src, type
     V* sm = smem + c * LS;
     V v[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = M::ld(src + sidx<N>(j + m * TL, col));
+    for (int m = 0; m < E; ++m) v[m] = src[sidx<N>(j + m * TL, col)];
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
         if (half == 1) conj_all(v);  // second round: B_y = conj(F_y(conj(.)))
@@ -581,7 +539,7 @@ __device__ __forceinline__ void col_tile(const typename vec2<T>::type* src, type
     // at 256^2 every tile gains from it)
     if constexpr (N < 512 || N / C >= 152) pdl_trigger();
 #pragma unroll
-    for (int m = 0; m < E; ++m) M::st(dst + sidx<N>(j + m * TL, col), v[m]);
+    for (int m = 0; m < E; ++m) dst[sidx<N>(j + m * TL, col)] = v[m];
 }
 
 // Row pass kernel of the march; with DIAG the block also reduces sum |U|^2 and
@@ -596,8 +554,7 @@ k_row_pass(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
     extern __shared__ __align__(16) unsigned char smraw[];
     T tsum = (T)0, tmax = (T)0;
     pdl_wait();
-    row_tile<T, N, RPB, DIAG, MemPlain>(src, dst, tw, sc, blockIdx.x * RPB, reinterpret_cast<V*>(smraw),
-                                        tsum, tmax);
+    row_tile<T, N, RPB, DIAG>(src, dst, tw, sc, blockIdx.x * RPB, reinterpret_cast<V*>(smraw), tsum, tmax);
     if constexpr (DIAG) block_partials<T>(tsum, tmax, partials);
 }
 
@@ -611,7 +568,7 @@ k_col_pass(const typename vec2<T>::type* src, typename vec2<T>::type* dst,
     using V = typename vec2<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     pdl_wait();
-    col_tile<T, N, C, MemPlain>(src, dst, tw, px, py, rot, blockIdx.x * C, reinterpret_cast<V*>(smraw));
+    col_tile<T, N, C>(src, dst, tw, px, py, rot, blockIdx.x * C, reinterpret_cast<V*>(smraw));
 }
 
 // Forward row transform S = F_x U (load prologue): src row-major, dst in the

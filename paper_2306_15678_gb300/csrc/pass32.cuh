@@ -214,7 +214,10 @@ static __device__ __noinline__ void screen_slow2(float re0, float re1, float im0
     cm1 = pk(k0, k1);
 }
 
-// U = v + v d, d = exp(s(|v|^2)) - 1 (kernels.cuh: apply_screen) on both lanes.
+// U = v + v d, d = exp(s(|v|^2)) - 1 = expm1(re) e^{i im} + (e^{i im} - 1), on both
+// lanes: the per-step change, not the field, carries the rounding of the factor, and
+// the whole of it is formed before a single rounding of v + v d (adding the small
+// second-order part after the first would lose it at every step, coherently).
 // Warp votes over both lanes of every thread pick a short polynomial (phases
 // within 1/32 rad) or the full one (within pi/4); otherwise each lane takes
 // the general scalar path of kernels.cuh.
