@@ -1033,21 +1033,29 @@ __device__ __forceinline__ C2 adj_value2(C2 v, C2 G, F2 u, F2 re, F2 im, F2 dre,
             fma(q, v.im, add(G.im, fma(dre, G.im, mul(neg(dim), G.re))))};
 }
 
-// Six per-thread pairs of FP32 sums (one per row) -> FP64 sums added into
-// acc[block][6], in a fixed order: each warp takes sums 0..5 in turn, its lanes every
-// 32nd thread's pair, then a shuffle tree.  The rows of a pair are joined in FP64 like
-// all others.  (A tree of FP64 shuffles in every warp is 30 FP64 additions per
-// thread: at 8192^2 a fifth of the kernel.)
+// The FP32 sums of a pair's two rows joined in FP64, like all others.  volatile: issued
+// here, between the transforms, where the slow FP64 pipe is idle and its latency passes
+// behind the second one (joined with the block's sums at the end instead, where nothing
+// overlaps with them at 8192^2, one block per SM: 606 -> 648 us per launch)
+__device__ __forceinline__ double join_rows(F2 g) {
+    double s;
+    asm volatile("add.rn.f64 %0, %1, %2;" : "=d"(s) : "d"((double)pr::lo(g)), "d"((double)pr::hi(g)));
+    return s;
+}
+// Six per-thread sums added into acc[block][6], in a fixed order: each warp takes sums
+// 0..5 in turn, its lanes every 32nd thread's value, then a shuffle tree.  (A tree of
+// FP64 shuffles in every warp is 30 FP64 additions per thread: at 8192^2 a fifth of the
+// kernel.)
 template <int THREADS>
-__device__ __forceinline__ void block_accumulate6_f32(const F2 (&g)[6], double* __restrict__ acc) {
-    __shared__ float2 red[6][THREADS];
+__device__ __forceinline__ void block_accumulate6_rows(const double (&g)[6], double* __restrict__ acc) {
+    __shared__ double red[6][THREADS];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = make_float2(pr::lo(g[q]), pr::hi(g[q]));
+    for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = g[q];
     __syncthreads();
     if constexpr (THREADS >= 32) {
         for (int q = (int)threadIdx.x >> 5; q < 6; q += THREADS / 32) {
             double s = 0.0;
-            for (int i = (int)threadIdx.x & 31; i < THREADS; i += 32) s += (double)red[q][i].x + (double)red[q][i].y;
+            for (int i = (int)threadIdx.x & 31; i < THREADS; i += 32) s += red[q][i];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if ((threadIdx.x & 31) == 0) acc[6 * blockIdx.x + q] += s;
@@ -1055,7 +1063,7 @@ __device__ __forceinline__ void block_accumulate6_f32(const F2 (&g)[6], double* 
     } else {
         for (int q = threadIdx.x; q < 6; q += THREADS) {
             double s = 0.0;
-            for (int i = 0; i < THREADS; ++i) s += (double)red[q][i].x + (double)red[q][i].y;
+            for (int i = 0; i < THREADS; ++i) s += red[q][i];
             acc[6 * blockIdx.x + q] += s;
         }
     }
@@ -1087,6 +1095,7 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
     F2 th[6];
 #pragma unroll
     for (int q = 0; q < 6; ++q) th[q] = pr::bc(0.0f);
+    double sum[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     auto pullback = [&]() {
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = pr::swp(v[m]);  // G_U = B_x G_S
@@ -1133,6 +1142,8 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
                 v[m0 + i] = adj_value2(w[i], v[m0 + i], u, re, im, dre, dim, ac, th);
             }
         }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) sum[q] = join_rows(th[q]);
     };
     if constexpr (MIR) {
         pr::fft_first<N, S>(v, sm, tab, t);
@@ -1148,7 +1159,7 @@ k_adj_row32(float4* gam, const float4* stash, const unsigned char* twb, AdjCoef<
     pdl_trigger();
 #pragma unroll
     for (int m = 0; m < E; ++m) UnitPlain::st(gam + row + j + m * T, v[m]);
-    block_accumulate6_f32<p_row_threads<N, 16>()>(th, acc);
+    block_accumulate6_rows<p_row_threads<N, 16>()>(sum, acc);
 }
 
 // Loss and seed (adjoint.cuh: k_loss_seed) on the unit layout, natural order (the
