@@ -701,19 +701,20 @@ def main():
                 h1.record(stream)
                 torch.cuda.synchronize(dev)
                 tt.append(h0.elapsed_time(h1))
-            # HBM sweeps of the implementation, bytes per point (FP32 grid): lens 196
-            # (readout 16, fluence 16, DFT pair and filter 80, labelling 28, centres 36,
-            # reload 16, plus the screen near the lenses), layer 104 (readout 16,
-            # spectrum 16, inverse DFT 32, phase 24, reload 16)
+            # HBM sweeps of the implementation, bytes per point (FP32 grid): lens 96
+            # (readout 16, row DFT of the fluence 16, column DFTs with the low-pass 16,
+            # row DFT to the real parts 12, labelling 20, reload 16; centres and screen
+            # near the lenses only), layer 80 (readout 16, inverse DFT 24: the draws are
+            # read within the cut-off only, phase 24, reload 16)
             pk_gbs = measured_peaks().get("hbm_gbs") or 6800.0
-            lens_gbs = 196.0 * n * n / (min(tl) / 1e3) / 1e9
-            turb_gbs = 104.0 * n * n / (min(tt) / 1e3) / 1e9
+            lens_gbs = 96.0 * n * n / (min(tl) / 1e3) / 1e9
+            turb_gbs = 80.0 * n * n / (min(tt) / 1e3) / 1e9
             lens_t = {"effective_lens_ms": min(tl), "lenses": nlens, "w_l_w_per_cm2": lens["w_l"],
                       "l_dif_cm2": lens["l_dif"], "turbulent_layer_ms": min(tt),
                       "lens_sweep_gbs": lens_gbs, "lens_hbm_frac": lens_gbs / pk_gbs,
                       "layer_sweep_gbs": turb_gbs, "layer_hbm_frac": turb_gbs / pk_gbs,
-                      "includes": "lens: readout, low-pass DFT pair, labelling, centres, ansatz sum, reload; "
-                                  "layer: readout, spectrum, inverse DFT pair, phase, reload"}
+                      "includes": "lens: readout, low-pass DFT sweeps, labelling, centres, ansatz sum, reload; "
+                                  "layer: readout, inverse DFT sweeps, phase, reload"}
 
         # ---- symmetric (Strang) steps on the same field: one more screen per row pass
         strang = None

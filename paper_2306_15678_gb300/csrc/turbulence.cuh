@@ -90,9 +90,10 @@ k_dft_rows(LD ld, ST st, const typename tab_of<T>::type* __restrict__ tw) {
 }
 // The same of every column, in place, and with LOWPASS the forward transform, the
 // separable factor fx[p] fy[q] on bin (q, p) (fy carries the 1/n^2 of the inverse
-// transforms) and the inverse transform in one sweep (2048^2: one sweep of 26 us for
-// two transforms of 22 and a filter of 12).  Blocks hold adjacent
-// columns with the column index fastest across the threads (coalesced sectors).
+// transforms) and the inverse transform in one sweep (2048^2, cold: 42 us for two
+// transforms of 22 and a filter of 12; it spills from 512^2 on, with two transforms
+// inlined at 64 registers).  Blocks hold adjacent columns with the column index fastest
+// across the threads (coalesced sectors).
 template <typename T, int N, bool LOWPASS>
 __global__ void __launch_bounds__(threads_per_line<T, N>() * dft_lines_per_block<T, N, true>(),
                                   min_blocks<threads_per_line<T, N>() * dft_lines_per_block<T, N, true>()>())
